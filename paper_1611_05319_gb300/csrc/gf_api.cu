@@ -61,6 +61,7 @@ struct gf_ctx {
         float ms;
     };
     std::vector<Tuned> tuned;
+    int max_clusters[3][5] = {};  // co-resident fill clusters by window (4, 5, 8) and size 1, 2, 4, 8, 16 (0: not asked yet)
 };
 
 static uint64_t tune_key(int n, const gf_frame *frames, const gf_params *p)
@@ -403,6 +404,11 @@ int gf_max_active_clusters(gf_ctx *ctx, float eps, int cluster_size)
 {
     if (!ctx) return -1;
     int rw = rw_for(eps);
+    // asked once per context, window and size: a property of the device
+    int *known = nullptr;
+    for (int i = 0; i < 5; i++)
+        if (cluster_size == 1 << i) known = &ctx->max_clusters[rw == 4 ? 0 : (rw == 5 ? 1 : 2)][i];
+    if (known && *known > 0) return *known;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cluster_size * 64);
     cfg.blockDim = dim3(32 * fill_warps(rw));
@@ -421,13 +427,27 @@ int gf_max_active_clusters(gf_ctx *ctx, float eps, int cluster_size)
         cudaGetLastError();
         return 0;
     }
+    if (known) *known = n;
     return n;
+}
+
+// Cluster size of a batch of n frames when neither set nor tuned: the largest with
+// which every frame has a cluster of its own at once, down to 4 CTAs (16 up to 7
+// frames, 8 up to 15).  A frame's fill is a chain of steps, which more CTAs shorten;
+// with fewer clusters than frames the last chains start late.  8 uneven 1080p frames:
+// 4.40 ms on clusters of 4, 3.25 on 8, 2.63 on 16 (7 at once); 16 frames of 512 x 512
+// alike: 0.91 ms on 4, 1.05 on 8 (15 at once).
+static int default_cluster_size(gf_ctx *ctx, float eps, int n)
+{
+    int cs = 16;
+    while (cs > 4 && gf_max_active_clusters(ctx, eps, cs) < n) cs >>= 1;
+    return cs;
 }
 
 static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const gf_params *prm,
                               gf_stats *dev_stats, cudaStream_t stream, cudaEvent_t ev0 = nullptr,
                               cudaEvent_t ev1 = nullptr, bool allow_graph = true, DevBuf *scratch = nullptr,
-                              cudaEvent_t wait_before_fill = nullptr)
+                              cudaEvent_t wait_before_fill = nullptr, bool allow_teams = true)
 {
     DevBuf &arena = scratch ? *scratch : ctx->arena;
     // ---- layout of the scratch arena
@@ -445,9 +465,12 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
         off_S[i] = pos; pos = align_up(pos + 4 * (size_t)ntiles[i], 256);
         off_L[i] = pos; pos = align_up(pos + 4 * (size_t)ntiles[i], 256);
     }
+    // what starts at zero, in one piece: hole counts, guided counts, front counts, teams
     const size_t off_holes = pos; pos = align_up(pos + 4 * (size_t)n, 256);
     const size_t off_gleft = pos; pos = align_up(pos + 4 * (size_t)n, 256);
     const size_t off_icnt = pos; pos = align_up(pos + 8 * (size_t)n, 256);
+    const size_t off_teams = pos; pos = align_up(pos + sizeof(TeamCtl) * (size_t)n, 256);
+    const size_t off_zero_end = pos;
     const size_t off_desc = pos; pos = align_up(pos + sizeof(FrameDev) * (size_t)n, 256);
     const size_t off_order = pos; pos = align_up(pos + 4 * (size_t)n, 256);
     const size_t off_cursor = pos; pos = align_up(pos + 8, 256);  // queue heads of the two launches
@@ -471,7 +494,7 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
                 }
             }
     }
-    if (cs == 0) cs = (n == 1) ? 16 : 4;  // before any autotuning: 16 CTAs for one frame, 4 per frame of a batch
+    if (cs == 0) cs = default_cluster_size(ctx, prm->eps, n);
     int maxc = gf_max_active_clusters(ctx, prm->eps, cs);
     while (maxc <= 0 && cs > 1) {
         cs /= 2;
@@ -490,13 +513,23 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
         else nc = std::min(nc, spare);
     }
     if (!split) sm = scs = snc = 0;
-    nc = std::max(1, std::min(nc, n - sm));
+    // clusters beyond the frames help the frames whose steps hold more tiles than
+    // their cluster has warps; no frame can use more than its tiles fill
+    int64_t useful = n - sm;
+    if (allow_teams && !split) {
+        const int unit = cs * fill_warps(rw);
+        useful = 0;
+        for (int i = 0; i < n; i++) useful += (ntiles[i] + unit - 1) / unit;
+    }
+    nc = (int)std::max<int64_t>(1, std::min<int64_t>(nc, useful));
     ctx->last_cluster_size = cs;
     ctx->last_n_clusters = nc;
     ctx->last_split_m = sm;
     ctx->last_split_cs = scs;
     ctx->last_split_nc = snc;
-    const int ncall = nc + snc;  // control blocks and work lists of both launches
+    if (nc == 1) allow_teams = false;
+    const int lists_main = std::min(nc, n - sm);
+    const int ncall = lists_main + snc;  // work lists of both launches
 
     const size_t off_lists = pos; pos = align_up(pos + 4 * (size_t)3 * list_cap * ncall, 256);
     gf_status st = ensure(ctx, arena, pos);
@@ -560,12 +593,16 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
     fp.frame_order = (int32_t *)(A + off_order);
     fp.frame_cursor = (int32_t *)(A + off_cursor);
     fp.lists = (int32_t *)(A + off_lists);
+    fp.lists_by_frame = nc > n - sm ? 1 : 0;
+    fp.teams = allow_teams ? (TeamCtl *)(A + off_teams) + sm : nullptr;
     build_tab(prm->eps, fp.tab);
     FillParams fpa = fp;  // the second launch: frame_order[0 .. sm)
     fpa.n_frames = sm;
     fpa.order_first = 0;
     fpa.frame_cursor = fp.frame_cursor + 1;
-    fpa.lists = fp.lists + (size_t)nc * 3 * list_cap;
+    fpa.lists = fp.lists + (size_t)lists_main * 3 * list_cap;
+    fpa.lists_by_frame = 0;
+    fpa.teams = allow_teams && snc > 1 ? (TeamCtl *)(A + off_teams) : nullptr;
 
     // graph key: everything the enqueued work depends on
     uint64_t key = 1469598103934665603ull;
@@ -624,10 +661,7 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
             e = cudaGetLastError();
         }
         if (e) break;
-        e = cudaMemsetAsync(A + off_holes, 0, 4 * (size_t)n, stream);
-        if (!e) e = cudaMemsetAsync(A + off_gleft, 0, 4 * (size_t)n, stream);
-        if (e) break;
-        e = cudaMemsetAsync(A + off_icnt, 0, 8 * (size_t)n, stream);
+        e = cudaMemsetAsync(A + off_holes, 0, off_zero_end - off_holes, stream);
         if (e) break;
         for (int i = 0; i < n && !e; i++) {
             const gf_frame &f = frames[i];
@@ -1739,7 +1773,7 @@ gf_status gf_fill_batched_host(gf_ctx *ctx, int n, const int32_t *H, const int32
             ctx->n_clusters = 0;
         }
         fs = enqueue_fill(ctx, q1 - q0, fr.data() + q0, params, (gf_stats *)(A + o_st) + q0, cs_st, nullptr, nullptr,
-                          false, &ctx->pipe_fill[c]);
+                          false, &ctx->pipe_fill[c], nullptr, false);
         ctx->cluster_size = keep.cs;
         ctx->n_clusters = keep.nc;
         if (fs != GF_OK) break;

@@ -390,17 +390,18 @@ __device__ bool warp_ready_fp64(const FillParams &p, const WarpSmem<RW> *ws, int
 constexpr int DS_LIST = 2048;
 struct Lists {
     int32_t *ds;    // [3][DS_LIST] in the first CTA's shared memory
-    int32_t *glob;  // [3][list_cap]; entries from DS_LIST on
+    int32_t *glob;  // [3][list_cap]; entries from nds on
     int cap;        // list_cap
+    int nds;        // DS_LIST, or 0 while a team of clusters fills the frame
 };
 __device__ __forceinline__ void list_put(const Lists &L, int slot, int pos, int32_t v)
 {
-    if (pos < DS_LIST) L.ds[slot * DS_LIST + pos] = v;
+    if (pos < L.nds) L.ds[slot * DS_LIST + pos] = v;
     else L.glob[(size_t)slot * L.cap + pos] = v;
 }
 __device__ __forceinline__ int32_t list_get(const Lists &L, int slot, int pos)
 {
-    return pos < DS_LIST ? ld(&L.ds[slot * DS_LIST + pos]) : ld(&L.glob[(size_t)slot * L.cap + pos]);
+    return pos < L.nds ? ld(&L.ds[slot * DS_LIST + pos]) : ld(&L.glob[(size_t)slot * L.cap + pos]);
 }
 
 struct WarpCounters {
@@ -414,8 +415,9 @@ struct WarpCounters {
 //    (one round trip); a lost claim leaves a skip marker (-1) in its slot;
 //  * deferred: the warp reserves slots only for the claims it won, once their
 //    atomics have returned (at its next tile), and writes the entries one tile
-//    later, so the list holds no skip markers.  Used when a step's list is longer
-//    than the cluster's warp count, where markers would be walked one by one.
+//    later, so the list holds no skip markers.  Used by teams and when a list with
+//    markers could be longer than the cluster's warp count, where they would be
+//    walked one by one.
 // The struct carries the claims of a warp's last tiles between those points.
 struct PendingClaims {
     unsigned m1;  // claims made, slots not yet reserved (warp-uniform lane mask)
@@ -450,7 +452,7 @@ __device__ __forceinline__ void claims_reserve(GroupCtl *ctl, PendingClaims &pc)
         const bool won = ((pc.m1 >> lane) & 1u) && pc.old1 < pc.k + 1;
         const unsigned wb = __ballot_sync(FULL, won);
         if (wb) {
-            if (lane == 0) pc.base2 = atomicAdd(&ctl->list_count[(pc.k + 1) % 3], __popc(wb));
+            if (lane == 0) pc.base2 = atomicAdd(&ctl->step[pc.k % 3].next, __popc(wb));
             pc.nt2 = pc.nt1;
             pc.old2 = INT32_MIN;
             pc.m2 = wb;
@@ -970,18 +972,27 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
             } else {
                 pc.m2 = bm;
                 pc.nt2 = nt;
-                if (lane == 0) pc.base2 = atomicAdd(&ctl->list_count[(k + 1) % 3], __popc(bm));
+                if (lane == 0) pc.base2 = atomicAdd(&ctl->step[k % 3].next, __popc(bm));
                 if (need) pc.old2 = atomicMax(&F.sched[nt], k + 1);
             }
         }
     }
 }
 
-// Adds a warp's counters of step k to slot k%3.  With `clear_next`, lane 0 of
-// the first warp of each CTA also clears the slot of step k+1 and the work-list
-// count of step k+2: their last readers passed the barrier of step k-1 and
-// their next writers start after the barrier of step k.
-__device__ __forceinline__ void flush_counters(GroupCtl *ctl, const WarpCounters &wc, int k, bool stall,
+__device__ __forceinline__ void clear_step(StepCtl *c)
+{
+    reinterpret_cast<int4 *>(c)[0] = make_int4(0, 0, 0, 0);
+    reinterpret_cast<int4 *>(c)[1] = make_int4(0, 0, 0, 0);
+}
+
+// Adds a warp's counters of step k to slot k%3.  With `clear_next`, lane 0 (of
+// the first warp of each CTA, in a team of the owner's first CTA) also clears
+// the slot of step k+1: its last readers passed the barrier of step k-1 and its
+// next writers start after the barrier of step k.  In a team (`acc` set) the
+// warps add into the CTA's shared counters, which team_sync sends on with one
+// atomic per CTA and counter: 256 warps or more adding to one L2 address would
+// take several microseconds a step.
+__device__ __forceinline__ void flush_counters(GroupCtl *ctl, int *acc, const WarpCounters &wc, int k, bool stall,
                                                bool clear_next)
 {
     const int lane = threadIdx.x & 31;
@@ -990,21 +1001,152 @@ __device__ __forceinline__ void flush_counters(GroupCtl *ctl, const WarpCounters
     // all lanes hold identical values except err (per lane)
     er = __reduce_or_sync(FULL, er);
     if (lane == 0) {
-        if (f) atomicAdd(&ctl->filled[s], f);
-        if (d) atomicAdd(&ctl->front_delta[s], d);
-        if (e && !stall) atomicAdd(&ctl->evals[s], e);  // Sigma_k |front_k| counts the evaluation pass only
-        if (er) atomicOr(&ctl->err[s], er);
-        if (rc) atomicAdd(&ctl->rechecks, rc);
-        if (clear_next) {
-            const int s1 = (k + 1) % 3;
-            ctl->cursor[s1] = 0;
-            ctl->filled[s1] = 0;
-            ctl->front_delta[s1] = 0;
-            ctl->evals[s1] = 0;
-            ctl->err[s1] = 0;
-            ctl->list_count[(k + 2) % 3] = 0;
+        if (acc) {
+            if (f) atomicAdd(&acc[0], f);
+            if (d) atomicAdd(&acc[1], d);
+            if (e && !stall) atomicAdd(&acc[2], e);
+            if (er) atomicOr(&acc[3], er);
+            if (rc) atomicAdd(&acc[4], rc);
+        } else {
+            StepCtl *c = &ctl->step[s];
+            if (f) atomicAdd(&c->filled, f);
+            if (d) atomicAdd(&c->front_delta, d);
+            if (e && !stall) atomicAdd(&c->evals, e);  // Sigma_k |front_k| counts the evaluation pass only
+            if (er) atomicOr(&c->err, er);
+            if (rc) atomicAdd(&ctl->rechecks, rc);
+        }
+        if (clear_next) clear_step(&ctl->step[(k + 1) % 3]);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Teams: several clusters on one frame
+// ---------------------------------------------------------------------------
+// A step of a frame with more tiles than its cluster has warps is bound by
+// throughput, and clusters hold 16 CTAs at most.  A cluster that finds the queue
+// empty therefore joins the running frame whose step is longest: it takes a
+// ticket (want), the frame's first cluster (its owner) answers the tickets taken
+// by the start of a step at that step's end (Admission), and the newcomers take
+// part from the next step on.  Only clusters that already run ask, so the
+// barrier never waits for a CTA that has no SM, and a plain launch does.  When a
+// step's list gets short, the members with the highest numbers leave again, and
+// with one cluster left the frame goes on under the hardware cluster barrier,
+// closed to joins.  Which warp processes a tile changes no result.
+//
+// Team barrier: every CTA adds one to a counter and polls it.  About 1 us a step
+// more than the cluster barrier, which is why a team is only as large as its
+// work list.  Measured against one cluster of 16 CTAs per frame, whole calls: a 4K
+// frame with a 400 x 400 blob (eps 4; first steps of 1,400 to 4,100 tiles on 256
+// warps) 4.47 -> 3.48 ms, a 2000 x 500 onion-order line problem (about 700 tiles a
+// step) 2.94 -> 1.69 ms, a 1500 x 1125 lattice-ball still 2.9 -> 1.8 ms, 32 uneven
+// 1080p frames (on clusters of 4) 4.83 -> 3.90 ms; thin cracks on one 1080p frame,
+// where few steps are that long, 1.32 -> 1.19 ms.
+constexpr unsigned TEAM_POLLS = 1u << 22;  // polls (about half a microsecond each) before a wait gives up
+
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
+{
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release(uint32_t *p, uint32_t v)
+{
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_volatile(const int32_t *p) { return *(const volatile int32_t *)p; }
+
+// Clusters that a step of n tiles keeps busy (`unit` warps each, one tile per warp).
+__device__ __forceinline__ int team_need(int n, int unit) { return max(1, (n + unit - 1) / unit); }
+
+// The barrier of a team's step (slot = step % 3): sends the CTA's counters, then
+// waits until `target` arrivals have been counted.  False when the wait gave up.
+__device__ __forceinline__ bool team_sync(TeamCtl *tc, int *acc, int *dead, int slot, uint32_t target)
+{
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        if (lane < 5) {
+            const int v = acc[lane];
+            acc[lane] = 0;
+            // err is 0 or 1 per CTA: a sum serves as well as an OR
+            if (v) atomicAdd(lane < 4 ? &tc->c.step[slot].filled + lane : &tc->c.rechecks, v);
+        }
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();
+            atomicAdd(&tc->bar, 1u);
+            unsigned n = 0;
+            while ((int32_t)(ld_acquire(&tc->bar) - target) < 0) {
+                if (++n >= TEAM_POLLS) {
+                    *dead = 1;
+                    break;
+                }
+            }
+            __threadfence();
         }
     }
+    __syncthreads();
+    return *dead == 0;
+}
+
+// What a cluster does next, in the shared memory of its first CTA: f >= 0 is a
+// queue position, -1 nothing is left; with help set the cluster is member
+// `member` of the frame's team.
+struct Role {
+    int32_t f, help, member, owner;
+    Admission adm;
+};
+
+// Looks for a running frame whose coming step has more tiles than its team has
+// warps, takes a ticket and waits for the answer; -1 when no frame wants help.
+// Called by the first warp of a cluster's first CTA.
+__device__ int team_find(const FillParams &p, int unit, Role *role)
+{
+    const int lane = threadIdx.x & 31;
+    for (unsigned tries = 0; tries < 4096u; tries++) {
+        // the frame that lacks most clusters
+        int best = 0, bf = -1, pending = 0;
+        for (int i = lane; i < p.n_frames; i += 32) {
+            const TeamCtl *tc = &p.teams[i];
+            const int load = ld_volatile(&tc->load);
+            if (load == 0) pending = 1;
+            if (load <= 0) continue;
+            const int asked = (int)(*(const volatile uint32_t *)&tc->want - *(const volatile uint32_t *)&tc->admitted);
+            const int lack = team_need(load, unit) - ld_volatile(&tc->team) - asked;
+            if (lack > best) {
+                best = lack;
+                bf = i;
+            }
+        }
+        const int top = __reduce_max_sync(FULL, best);
+        if (top <= 0) {
+            // frames taken from the queue but not started yet may want help in a moment
+            if (__any_sync(FULL, pending) && tries < 64u) {
+                __nanosleep(500);
+                continue;
+            }
+            return -1;
+        }
+        const int src = __ffs(__ballot_sync(FULL, best == top)) - 1;
+        bf = __shfl_sync(FULL, bf, src);
+        int got = 0;
+        if (lane == 0) {
+            TeamCtl *tc = &p.teams[bf];
+            const uint32_t ticket = atomicAdd(&tc->want, 1u);
+            for (unsigned n = 0; n < TEAM_POLLS; n++) {
+                if ((int32_t)(ld_acquire(&tc->admitted) - ticket) > 0) {
+                    role->adm = tc->adm;
+                    role->owner = tc->owner;
+                    role->member = role->adm.first_member + (int)ticket - role->adm.first_ticket;
+                    got = 1;
+                    break;
+                }
+                if (ld_volatile(&tc->load) < 0) break;  // over, or closed
+            }
+        }
+        if (__shfl_sync(FULL, got, 0)) return bf;
+    }
+    return -1;
 }
 
 // Every warp of the cluster visits the frame's tiles (32 at a time); the mode
@@ -1044,14 +1186,15 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
     // CTA's shared memory
     __shared__ GroupCtl s_ctl;
     __shared__ int32_t s_lists[3 * DS_LIST];
-    GroupCtl *ctl = cluster.map_shared_rank(&s_ctl, 0);
+    __shared__ Role s_role[2];
+    __shared__ int s_acc[5];   // the CTA's step counters while it is in a team
+    __shared__ int s_dead;     // a team barrier's wait gave up
+    GroupCtl *const ds_ctl = cluster.map_shared_rank(&s_ctl, 0);
+    const Role *const ds_role = cluster.map_shared_rank(s_role, 0);
     Lists lists;
     lists.ds = cluster.map_shared_rank(s_lists, 0);
-    lists.glob = p.lists + (size_t)cid * 3 * p.list_cap;
     lists.cap = p.list_cap;
-    const int gw = (threadIdx.x >> 5) * csize + crank;  // interleave CTAs
-    const int nw = csize * fill_warps(RW);
-    const bool leader = crank == 0 && threadIdx.x == 0;
+    const int unit = csize * fill_warps(RW);  // warps of a cluster
     const bool rescan = (p.flags & GF_FLAG_RESCAN) != 0;
     for (int i = threadIdx.x; i < p.tab.nsp; i += blockDim.x) {
         g_stab[i] = make_float4(p.tab.n_f[i], p.tab.m_f[i], p.tab.invd[i], fabsf(p.tab.m_f[i]));
@@ -1067,55 +1210,170 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
         }
     }
     if ((threadIdx.x & 31) == 0) ws->col[WarpSmem<RW>::WS * WarpSmem<RW>::WS] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (threadIdx.x < 5) s_acc[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_dead = 0;
     __syncthreads();
 
     for (int it = 0;; it++) {
         cluster.sync();  // everyone is done with the previous frame's counters
-        if (leader) {
-            int f = atomicAdd(p.frame_cursor, 1);
-            ctl->cur_frame[it & 1] = f;
-            for (int i = 0; i < 3; i++) {
-                ctl->list_count[i] = 0;
-                ctl->cursor[i] = 0;
-                ctl->filled[i] = 0;
-                ctl->front_delta[i] = 0;
-                ctl->evals[i] = 0;
-                ctl->err[i] = 0;
+        if (crank == 0 && threadIdx.x < 32) {
+            Role *role = &s_role[it & 1];
+            int f = 0, help = 0;
+            if (threadIdx.x == 0) {
+                f = atomicAdd(p.frame_cursor, 1);
+                for (int i = 0; i < 3; i++) clear_step(&s_ctl.step[i]);
+                s_ctl.rechecks = 0;
             }
-            ctl->rechecks = 0;
+            f = __shfl_sync(FULL, f, 0);
+            if (f >= p.n_frames) {
+                f = p.teams ? team_find(p, unit, role) : -1;
+                help = 1;
+            }
+            if (threadIdx.x == 0) {
+                role->f = f;
+                role->help = help;
+            }
         }
         cluster.sync();
-        const int f = ld(&ctl->cur_frame[it & 1]);
-        if (f >= p.n_frames) break;
-        if (threadIdx.x == 0) s_frame = p.frames[p.frame_order[p.order_first + f]];
+        const Role *role = ds_role + (it & 1);
+        const int f = role->f;
+        if (f < 0) break;
+        const bool own = role->help == 0;
+        const bool leader = own && crank == 0 && threadIdx.x == 0;
+        if (threadIdx.x == 0) {
+            s_frame = p.frames[p.frame_order[p.order_first + f]];
+            __threadfence();  // a joining CTA's L1 holds nothing of the frame's earlier steps
+        }
         __syncthreads();
         const FrameDev &F = s_frame;
+        TeamCtl *const tc = p.teams ? &p.teams[f] : nullptr;
+        lists.glob = p.lists + (size_t)(p.lists_by_frame ? f : (own ? cid : role->owner)) * 3 * p.list_cap;
 
-        long long n_front = ld(&F.init_count[1]);
+        // uniform over the clusters that fill the frame: its team of `team` clusters,
+        // of which this one is number `member`; bar: arrivals the team's barrier has
+        // counted when the running step ends; admitted: tickets answered
+        int team = 1, member = 0, admitted = 0;
+        uint32_t bar = 0;
+        bool open = p.teams != nullptr;
+        GroupCtl *ctl = ds_ctl;
+        int gw, nw;
+        auto shape = [&]() {
+            gw = ((threadIdx.x >> 5) * team + member) * csize + crank;  // interleave CTAs
+            nw = team * unit;
+            ctl = team > 1 ? &tc->c : ds_ctl;
+            lists.nds = team > 1 ? 0 : DS_LIST;
+        };
+        // adds the step's counters and waits for everyone; `leave`: arrivals owed by
+        // CTAs that left the team at the end of the last step
+        int leave = 0;
+        auto finish = [&](const WarpCounters &w, int k, bool stall, bool clear) -> bool {
+            flush_counters(ctl, team > 1 ? s_acc : nullptr, w, k, stall, clear);
+            if (team == 1) {
+                cluster.sync();
+                return true;
+            }
+            bar += (uint32_t)(team * csize + leave);
+            leave = 0;
+            return team_sync(tc, s_acc, &s_dead, k % 3, bar);
+        };
+
+        long long n_front = 0;
         long long filled_tot = 0, evals_tot = 0, max_front = 0;
         int stalls = 0, status = GF_OK;
         int k = 0;
         const int max_shells = F.max_shells;
-        // the length and the first item of the current step's work list are loaded
-        // ahead, together with the previous step's counters
-        int n_cur = ld(&F.init_count[0]);
-        int t0_cur = gw < n_cur ? ld(&F.init_list[gw]) : -1;
+        int n_cur = 0;
         // eq. ready2 (GF_FLAG_DATA): phase 1 while hole pixels with g != 0 remain and
         // some front pixel is ready under the data term; `reval`: this step tests every
         // front pixel with eq. ready (the tracked front was built under phase 1)
         bool phase1 = (p.flags & GF_FLAG_DATA) != 0;
         int data_switch = -1;
         bool reval = false;
-        if (phase1 && ld(F.gleft) == 0) {
-            phase1 = false;
-            data_switch = 0;
+        if (own) {
+            n_front = ld(&F.init_count[1]);
+            n_cur = ld(&F.init_count[0]);
+            if (phase1 && ld(F.gleft) == 0) {
+                phase1 = false;
+                data_switch = 0;
+            }
+        } else {
+            const Admission &adm = role->adm;
+            member = role->member;
+            team = adm.team;
+            k = adm.k;
+            n_cur = adm.n_cur;
+            n_front = adm.n_front;
+            phase1 = adm.phase1 != 0;
+            reval = adm.reval != 0;
+            bar = adm.bar;
+            admitted = adm.first_ticket + (adm.team - adm.first_member);
         }
+        // tells the clusters whose tickets up to `upto` were answered that they are in
+        // the team from step k on
+        auto admit = [&](int upto, int team_old) {
+            tc->adm.first_ticket = admitted;
+            tc->adm.first_member = team_old;
+            tc->adm.team = team;
+            tc->adm.k = k;
+            tc->adm.n_cur = n_cur;
+            tc->adm.phase1 = phase1 ? 1 : 0;
+            tc->adm.reval = reval ? 1 : 0;
+            tc->adm.bar = bar;
+            tc->adm.n_front = n_front;
+            tc->team = team;
+            __threadfence();
+            st_release(&tc->admitted, (uint32_t)upto);
+        };
+        const int sweep_load = max(1, F.ntiles / 8);  // rescan: tiles swept 32 at a time by a warp
+        if (own && open) {
+            const int load = rescan ? sweep_load : max(n_cur, 1);
+            const int need = team_need(load, unit);
+            if (leader) {
+                tc->owner = cid;
+                tc->team = 1;
+                __threadfence();
+                *(volatile int32_t *)&tc->load = load;
+            }
+            // clusters without a frame of their own are already looking for one: a
+            // moment's wait lets them take part in the first step, the longest of most fills
+            const int spare = min(need - 1, (int)(gridDim.x / csize) - p.n_frames);
+            if (spare > 0) {
+                if (leader) {
+                    const long long t0 = clock64();
+                    uint32_t w;
+                    do {
+                        w = *(volatile uint32_t *)&tc->want;
+                    } while ((int)w < spare && clock64() - t0 < 8000);
+                    s_ctl.step[2].join = (int)w;
+                }
+                cluster.sync();
+                const int w = ld(&ds_ctl->step[2].join);
+                if (w > 0) {
+                    team = 1 + w;
+                    if (leader) admit(w, 1);
+                    admitted = w;
+                }
+            }
+        }
+        shape();
+        // the first item of the current step's work list is loaded ahead, together with
+        // the previous step's counters
+        int t0_cur = -1;
+        if (gw < n_cur) t0_cur = k == 0 ? ld(&F.init_list[gw]) : list_get(lists, k % 3, gw);
         for (;;) {
             const int slot = k % 3;
             WarpCounters wc = {0, 0, 0, 0, 0};
             PendingClaims pc;
             pc.m1 = 0u;
             pc.m2 = 0u;
+            int asked = 0;
+            if (leader && open) asked = (int)*(volatile uint32_t *)&tc->want;
+            const bool more = n_cur > nw;
+            // lost claims leave markers, up to 1.5 per tile: where they could make the next
+            // list longer than the warps, and a second round of it, they are avoided
+            // (a 1080p step of about 180 tiles on 256 warps took 13 us with a list of 400
+            // entries against 9.5 us with a compact one)
+            const bool defer = team > 1 || 5 * n_cur > 2 * nw;
             if (rescan) {
                 sweep_tiles<RW, RESCAN>(p, F, ws, ctl, lists, k, gw, nw, wc, pc, phase1);
             } else if (reval) {
@@ -1129,31 +1387,33 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
                 // processed), so uneven tiles do not leave warps idle at the barrier.
                 // Negative items are claims lost to another tile.
                 const bool lane0 = (threadIdx.x & 31) == 0;
-                const bool more = n > nw;
                 int pre = 0;
-                if (lane0 && more) pre = atomicAdd(&ctl->cursor[slot], 1);
+                if (lane0 && more) pre = atomicAdd(&ctl->step[slot].cursor, 1);
                 const int t0 = gw < n ? t0_cur : -1;
-                if (t0 >= 0) process_tile<RW, NORMAL>(p, F, ws, ctl, lists, t0, k, 0ull, wc, pc, more, phase1);
+                if (t0 >= 0) process_tile<RW, NORMAL>(p, F, ws, ctl, lists, t0, k, 0ull, wc, pc, defer, phase1);
                 if (more) {
                     int nxt = nw + __shfl_sync(FULL, pre, 0);
                     while (nxt < n) {
                         const int t = k == 0 ? ld(&F.init_list[nxt]) : list_get(lists, slot, nxt);
-                        if (lane0) pre = atomicAdd(&ctl->cursor[slot], 1);
-                        if (t >= 0) process_tile<RW, NORMAL>(p, F, ws, ctl, lists, t, k, 0ull, wc, pc, more, phase1);
+                        if (lane0) pre = atomicAdd(&ctl->step[slot].cursor, 1);
+                        if (t >= 0) process_tile<RW, NORMAL>(p, F, ws, ctl, lists, t, k, 0ull, wc, pc, defer, phase1);
                         nxt = nw + __shfl_sync(FULL, pre, 0);
                     }
                 }
             }
             claims_drain(p, ctl, lists, pc, wc);
-            flush_counters(ctl, wc, k, false, threadIdx.x < 32);
-            cluster.sync();
+            if (leader && open) ctl->step[slot].join = asked;
+            if (!finish(wc, k, false, threadIdx.x < 32 && (team == 1 || (own && crank == 0)))) {
+                status = GF_ERR_TIMEOUT;
+                break;
+            }
             // one round trip: this step's counters and the next step's list
             const int s3n = (k + 1) % 3;
-            int filled = ld(&ctl->filled[slot]);
-            int dlt = ld(&ctl->front_delta[slot]);
-            const int ev = ld(&ctl->evals[slot]);
-            const int er = ld(&ctl->err[slot]);
-            int n_next = ld(&ctl->list_count[s3n]);
+            const int4 c0 = ld(reinterpret_cast<const int4 *>(&ctl->step[slot]));
+            const int2 c1 = ld(reinterpret_cast<const int2 *>(&ctl->step[slot].next));
+            int filled = c0.x, dlt = c0.y, n_next = c1.x;
+            const int ev = c0.z, er = c0.w;
+            const int join = open ? c1.y : 0;
             int t0_next = gw < p.list_cap ? list_get(lists, s3n, gw) : -1;  // used only if gw < n_next
             const int gleft = phase1 ? ld(F.gleft) : -1;
             evals_tot += ev;
@@ -1172,12 +1432,14 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
                 WarpCounters wr = {0, 0, 0, 0, 0};
                 sweep_tiles<RW, REVAL>(p, F, ws, ctl, lists, k, gw, nw, wr, pc);
                 claims_drain(p, ctl, lists, pc, wr);
-                flush_counters(ctl, wr, k, true, false);
-                cluster.sync();
-                filled = ld(&ctl->filled[slot]);
-                dlt = ld(&ctl->front_delta[slot]);
-                const int er1 = ld(&ctl->err[slot]);
-                n_next = ld(&ctl->list_count[s3n]);
+                if (!finish(wr, k, true, false)) {
+                    status = GF_ERR_TIMEOUT;
+                    break;
+                }
+                filled = ld(&ctl->step[slot].filled);
+                dlt = ld(&ctl->step[slot].front_delta);
+                const int er1 = ld(&ctl->step[slot].err);
+                n_next = ld(&ctl->step[slot].next);
                 t0_next = gw < p.list_cap ? list_get(lists, s3n, gw) : -1;
                 if (er1) {
                     status = GF_ERR_INTERNAL;
@@ -1200,13 +1462,15 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
                 WarpCounters ws2 = {0, 0, 0, 0, 0};
                 sweep_tiles<RW, STALL>(p, F, ws, ctl, lists, k, gw, nw, ws2, pc);
                 claims_drain(p, ctl, lists, pc, ws2);
-                flush_counters(ctl, ws2, k, true, false);
-                cluster.sync();
-                const int sf = ld(&ctl->filled[slot]);
-                const int dlt2 = ld(&ctl->front_delta[slot]);
-                const int er2 = ld(&ctl->err[slot]);
+                if (!finish(ws2, k, true, false)) {
+                    status = GF_ERR_TIMEOUT;
+                    break;
+                }
+                const int sf = ld(&ctl->step[slot].filled);
+                const int dlt2 = ld(&ctl->step[slot].front_delta);
+                const int er2 = ld(&ctl->step[slot].err);
                 // the stall fills appended claims to the next step's list
-                n_next = ld(&ctl->list_count[s3n]);
+                n_next = ld(&ctl->step[slot].next);
                 t0_next = gw < p.list_cap ? list_get(lists, s3n, gw) : -1;
                 if (er2) {
                     status = GF_ERR_INTERNAL;
@@ -1221,6 +1485,9 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
                 n_front += dlt;
             }
             filled_tot += fk;
+            // without deferred claims the list holds markers of lost ones; its tiles are
+            // then about as many as this step's, at most one per warp
+            const int load = rescan ? sweep_load : (defer ? n_next : min(n_next, nw));
             n_cur = n_next;
             t0_cur = t0_next;
             k++;
@@ -1228,8 +1495,60 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
                 status = GF_ERR_NO_PROGRESS;
                 break;
             }
+            if (!open) continue;
+            // the team of the next step: with the clusters that asked to join, or
+            // without those that its list does not keep busy
+            const int need = team_need(load, unit);
+            const int team_old = team;
+            if (join > admitted) team += join - admitted;
+            else if (need < team) team = need;
+            if (team == team_old) {
+                if (leader) *(volatile int32_t *)&tc->load = max(load, 1);
+                continue;
+            }
+            const int nh = min(n_cur, DS_LIST);  // the list's head moves between shared and global memory
+            int32_t *hg = lists.glob + (size_t)s3n * p.list_cap, *hs = lists.ds + s3n * DS_LIST;
+            if (team > team_old) {
+                if (team_old == 1) {
+                    for (int i = crank * blockDim.x + threadIdx.x; i < nh; i += csize * blockDim.x) hg[i] = hs[i];
+                    cluster.sync();
+                }
+                if (leader) {
+                    admit(join, team_old);
+                    *(volatile int32_t *)&tc->load = max(load, 1);
+                }
+                admitted = join;
+            } else if (team > 1) {
+                // a CTA that leaves still counts at the next barrier, so that nobody clears
+                // the counters it has read until it has
+                leave = (team_old - team) * csize;
+                if (leader) {
+                    tc->team = team;
+                    *(volatile int32_t *)&tc->load = max(load, 1);
+                }
+                if (member >= team) {
+                    __syncthreads();
+                    if (threadIdx.x == 0) {
+                        __threadfence();
+                        atomicAdd(&tc->bar, 1u);
+                    }
+                    break;
+                }
+            } else {
+                // one cluster goes on alone, under the cluster barrier
+                open = false;
+                if (leader) *(volatile int32_t *)&tc->load = -1;
+                if (member > 0) break;
+                if (leader)
+                    for (int i = 0; i < 3; i++) clear_step(&s_ctl.step[i]);
+                for (int i = crank * blockDim.x + threadIdx.x; i < nh; i += csize * blockDim.x) hs[i] = hg[i];
+                cluster.sync();
+            }
+            shape();
+            t0_cur = gw < n_cur ? list_get(lists, s3n, gw) : -1;
         }
         if (leader) {
+            if (tc) *(volatile int32_t *)&tc->load = -1;
             const int holes = ld(F.holes);
             gf_stats st;
             st.shells = k;
@@ -1238,7 +1557,7 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
             st.evaluations = evals_tot;
             st.max_front = max_front;
             st.holes = holes;
-            st.rechecks = ld(&ctl->rechecks);
+            st.rechecks = s_ctl.rechecks + (tc ? ld(&tc->c.rechecks) : 0);
             st.data_switch = data_switch;
             st.reserved = 0;
             if (status == GF_OK && filled_tot < holes) status = GF_INCOMPLETE;
@@ -1246,6 +1565,7 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
             *F.stats = st;
         }
         __syncthreads();
+        if (s_dead) return;  // a wait gave up: no further barrier can be relied on
     }
     cp_async_wait_all();  // window copies of a last tile that had no candidates
     // no CTA leaves while another may still read its shared memory (the control

@@ -93,23 +93,53 @@ struct FrameDev {
     int32_t *gleft;               // GF_FLAG_DATA: unfilled hole pixels with g != 0 (init kernel, then fills)
 };
 
+// The counters of one step: two 16-byte loads after the step's barrier.
+struct alignas(16) StepCtl {
+    int32_t filled;               // fills (evaluation pass, then stall pass if any)
+    int32_t front_delta;          // net change of the front size
+    int32_t evals;                // front pixels evaluated (evaluation pass only)
+    int32_t err;
+    int32_t next;                 // length of the next step's work list, built by this step's claims
+    int32_t join;                 // tickets of the frame's team (TeamCtl::want) seen when the step began
+    int32_t cursor;               // hand-out cursor of the items beyond the warp count
+    int32_t pad;
+};
+
 // Per-cluster control block (in the shared memory of the cluster's first CTA,
-// used by every CTA through distributed shared memory).  Counters are indexed by
-// the step that writes them (mod 3) so that no counter is reset while another
-// CTA of the cluster may still read it.
+// used by every CTA through distributed shared memory).  Step s uses slot s%3:
+// during step s the slot of step s+1 is cleared, so a slot is never cleared
+// while a warp of the cluster may still read it.
 struct GroupCtl {
-    // Per-step counters live in slot s%3 for step s.  During step s the slot of
-    // step s+1 (and the work-list count of step s+2) is cleared, so a slot is
-    // never cleared while a warp of the cluster may still read it.
-    int32_t list_count[3];        // work list consumed by step s lives in slot s%3
-    int32_t cursor[3];            // hand-out cursor of the items of step s beyond the warp count
-    int32_t filled[3];            // fills of step s (evaluation pass, then stall pass if any)
-    int32_t front_delta[3];       // net change of the front size during step s
-    int32_t evals[3];             // front pixels evaluated at step s (evaluation pass only)
-    int32_t err[3];
+    StepCtl step[3];
     int32_t rechecks;             // FP64 re-checks of the current frame (statistics only)
-    int32_t cur_frame[2];
     int32_t pad[3];
+};
+
+// What a cluster that joins a running frame needs to know, besides the tickets
+// and members it is told apart by.
+struct Admission {
+    int32_t first_ticket;         // the tickets first_ticket .. are members first_member ..
+    int32_t first_member;
+    int32_t team;                 // clusters from step k on
+    int32_t k;                    // the next step
+    int32_t n_cur;                // its work list's length
+    int32_t phase1, reval;
+    uint32_t bar;                 // arrivals that the team's barrier has counted
+    int64_t n_front;
+};
+
+// Per-frame control block in global memory for a frame that several clusters
+// fill (zero at launch).  The polled words and the counters sit in 128-byte
+// lines of their own.
+struct alignas(128) TeamCtl {
+    GroupCtl c;                   // the step counters while the team has several clusters
+    alignas(128) uint32_t bar;    // arrivals at the team's barrier, one per CTA and step
+    alignas(128) uint32_t want;   // tickets handed out to clusters that ask to join
+    alignas(128) uint32_t admitted;  // tickets answered (adm holds the last answer)
+    int32_t load;                 // 0 not started, > 0 tiles of the coming step, < 0 closed to joins
+    int32_t team;                 // clusters filling the frame
+    int32_t owner;                // cluster that took the frame from the queue
+    Admission adm;
 };
 
 struct FillParams {
@@ -124,7 +154,9 @@ struct FillParams {
     FrameDev *frames;
     int32_t *frame_order;         // all frames of the request, largest hole first (device)
     int32_t *frame_cursor;        // this launch's work queue head
-    int32_t *lists;               // [n_clusters][3][list_cap]
+    int32_t *lists;               // [n_clusters][3][list_cap], or by queue position with lists_by_frame
+    int32_t lists_by_frame;       // more clusters than frames: [n_frames][3][list_cap]
+    TeamCtl *teams;               // [n_frames], by queue position; null: every frame stays with one cluster
     SampleTab tab;
 };
 
