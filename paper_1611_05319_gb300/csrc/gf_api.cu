@@ -297,7 +297,7 @@ gf_status gf_create(gf_ctx **out, int device)
     }
     for (int rw : {4, 5, 8}) {
         const void *k = fill_kernel_ptr(rw);
-        size_t smem = warp_smem(rw) * fill_warps(rw);
+        size_t smem = warp_smem(rw) * FILL_WARPS;
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) {
@@ -411,8 +411,8 @@ int gf_max_active_clusters(gf_ctx *ctx, float eps, int cluster_size)
     if (known && *known > 0) return *known;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cluster_size * 64);
-    cfg.blockDim = dim3(32 * fill_warps(rw));
-    cfg.dynamicSmemBytes = warp_smem(rw) * fill_warps(rw);
+    cfg.blockDim = dim3(32 * FILL_WARPS);
+    cfg.dynamicSmemBytes = warp_smem(rw) * FILL_WARPS;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = cluster_size;
@@ -517,7 +517,7 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
     // their cluster has warps; no frame can use more than its tiles fill
     int64_t useful = n - sm;
     if (allow_teams && !split) {
-        const int unit = cs * fill_warps(rw);
+        const int unit = cs * FILL_WARPS;
         useful = 0;
         for (int i = 0; i < n; i++) useful += (ntiles[i] + unit - 1) / unit;
     }
@@ -630,8 +630,8 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(nc * cs));
-    cfg.blockDim = dim3(32 * fill_warps(rw));
-    cfg.dynamicSmemBytes = warp_smem(rw) * fill_warps(rw);
+    cfg.blockDim = dim3(32 * FILL_WARPS);
+    cfg.dynamicSmemBytes = warp_smem(rw) * FILL_WARPS;
     cfg.stream = stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;

@@ -55,14 +55,13 @@ __device__ __forceinline__ T ld(const T *p)
     return *p;
 }
 
-// The sample table of the fill kernel in shared memory: (n, m, 1/|(n, m)|, |m|)
-// in grouped order, padded to a multiple of 32 (one 16-byte load per sample; the
-// lanes of a pixel read different entries, which the constant cache would
-// serialise).
-__shared__ float4 g_stab[MAX_SAMPLES];
-// The same samples as mirror pairs {(n, m), (-n, -m)}: one entry per pair,
-// (n, m, 1/|(n, m)|, |m| as int bits) with m < 0, or m = 0 and n < 0.
-__shared__ float4 g_pair[MAX_SAMPLES / 2];
+// The ball's samples in shared memory as mirror pairs {(n, m), (-n, -m)}, one entry
+// per pair, with m < 0, or m = 0 and n < 0: (n, n, m, m), ready for two-wide
+// arithmetic, and (1/|(n, m)|, code) with code = |m| | (n + 8) << 8 | (m + 8) << 16.
+// (The lanes of a pixel read different entries, which the constant cache would
+// serialise.)
+__shared__ float4 g_pos[MAX_SAMPLES / 2];
+__shared__ float2 g_wt[MAX_SAMPLES / 2];
 
 // ---------------------------------------------------------------------------
 // init
@@ -383,6 +382,342 @@ __device__ bool warp_ready_fp64(const FillParams &p, const WarpSmem<RW> *ws, int
     return __ddiv_rn(S_rd, S_all) > p.c64;
 }
 
+// Lanes per front pixel of a tile with n front pixels (n capped at 17): as many as
+// the warp has for them, and ceil(256 / lanes), with which (lane * y) >> 8 is lane /
+// lanes.  Any count of lanes goes: 9 pixels get 3 lanes each and 5 iterations over
+// the 14 pairs of eps = 3 where powers of two gave 2 lanes and 7.
+__constant__ int2 c_lanes[18] = {{32, 8},  {32, 8},  {16, 16}, {10, 26}, {8, 32},   {6, 43},
+                                 {5, 52},  {4, 64},  {4, 64},  {3, 86},  {3, 86},   {2, 128},
+                                 {2, 128}, {2, 128}, {2, 128}, {2, 128}, {2, 128},  {1, 256}};
+
+// Two FP32 operations in one instruction (each correctly rounded, as the scalar ones).
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi)
+{
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v)
+{
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// Sums over a pixel's readable samples.  The weights' sum is kept with its rounding
+// error (lo): the same pattern of readable samples meets a front again and again, and
+// an error of the divisor of half an ulp, the same each time, would add up over a
+// long chain of shells (a 4K frame with 250 shells was 3.8e-7 off its values in 64
+// bits, and is 3e-8 off now).
+struct Acc {
+    unsigned long long xy, zw;  // colours, two channels a word
+    float s, lo;                // weights
+};
+// s + w, its rounding error added to lo
+__device__ __forceinline__ void weight_add(float &s, float &lo, float w)
+{
+    const float t = __fadd_rn(s, w), b = __fsub_rn(t, s);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(w, b)));
+    s = t;
+}
+__device__ __forceinline__ void acc_add(Acc &a, unsigned long long w, const ulonglong2 &c)
+{
+    a.xy = fma2(w, c.x, a.xy);
+    a.zw = fma2(w, c.y, a.zw);
+}
+
+// The set of the pixels `pix` of the lanes with `in` (every lane gets it): two warp
+// reductions, where 64-bit atomics on a shared word would be retried lane by lane.
+__device__ __forceinline__ unsigned long long pixel_mask(bool in, int pix)
+{
+    const uint32_t bit = in ? 1u << (pix & 31) : 0u;
+    const uint32_t lo = __reduce_or_sync(FULL, pix < 32 ? bit : 0u);
+    const uint32_t hi = __reduce_or_sync(FULL, pix < 32 ? 0u : bit);
+    return (unsigned long long)hi << 32 | lo;
+}
+
+// The readable bits around a pixel as one word (R <= 3): rows -3 .. 3, 8 columns -3
+// .. 4 each, bit 8 (dy + 3) + dx + 3.
+template <int RW>
+__device__ __forceinline__ unsigned long long around(const WarpSmem<RW> *ws, int px, int py)
+{
+    uint32_t lo = 0, hi = 0;
+#pragma unroll
+    for (int r = 0; r < 4; r++) lo |= ((ws->rowmask[py + RW - 3 + r] >> (px + RW - 3)) & 0xffu) << (8 * r);
+#pragma unroll
+    for (int r = 0; r < 3; r++) hi |= ((ws->rowmask[py + RW + 1 + r] >> (px + RW - 3)) & 0xffu) << (8 * r);
+    return (unsigned long long)hi << 32 | lo;
+}
+
+// The rotated ball of one pixel, over the mirror pairs j, j + G, ...: readable
+// weights (unnormalised), whether any sample is readable, weighted colours.
+//
+// Negation is exact and commutes with every rounding of the rotation and of the
+// snap, so the second sample's offset is the exact negative of the first's; the
+// pair shares its rotation, snap, floor and weights, and each tap of the second
+// sample is the first's tap reflected through the pixel, with the same bilinear
+// weight.  Taps of zero weight and the taps of unreadable samples are read from the
+// window's zero entry (an unreadable pixel's colour may be anything, and 0 * NaN is
+// NaN).
+//
+// Bound by the dependent instructions of an iteration, so: two-wide arithmetic for
+// the rotation and the colours; rounding to the lattice by adding 1.5 * 2^23 (the
+// difference d to the nearest integer is exact, and floor and fraction follow from
+// its sign) instead of the conversion unit; BITS: the readability of a sample's
+// cell as one shift and one mask of a register word, the mirrored sample's with the
+// same shift and mask of the reversed word, instead of four shared loads.  BITS
+// needs R <= 3 and a snap that covers the rotation's rounding, |offset| <= R.
+// Measured (cycles of a tile's sample passes, one 1080p frame, eps 3): 9 to 16 front
+// pixels 8,200 -> 6,100, 17 and more 13,100 -> 8,900, an iteration 620 -> 450.
+template <int RW, bool BITS>
+__device__ __forceinline__ void rotated_pairs(const FillParams &p, const WarpSmem<RW> *ws, const float *eg, int pix, int j,
+                                              int G, float ch, float sh, bool &any_, Acc &acc_)
+{
+    constexpr int WS = WarpSmem<RW>::WS, ZI = WS * WS;
+    const int px = pix & 7, py = pix >> 3;
+    const ulonglong2 *col = reinterpret_cast<const ulonglong2 *>(ws->col);
+    const int cx = px + RW, cy = py + RW, c0 = cy * WS + cx;
+    const unsigned long long c1 = pack2(ch, sh), c2 = pack2(-sh, ch);
+    const unsigned long long big = pack2(12582912.0f, 12582912.0f), nbig = pack2(-12582912.0f, -12582912.0f);
+    const unsigned long long neg1 = pack2(-1.0f, -1.0f);
+    const float tau = p.tau;
+    const int npair = p.tab.ns >> 1;
+    unsigned long long near = 0, rnear = 0;
+    if (BITS) {
+        near = around<RW>(ws, px, py);
+        rnear = __brevll(near);
+    }
+    bool any = false;
+    Acc acc = {0ull, 0ull, 0.f, 0.f};
+#pragma unroll 1
+    for (int q = j; q < npair; q += G) {
+        const ulonglong2 nm = *reinterpret_cast<const ulonglong2 *>(&g_pos[q]);  // (n, n), (m, m)
+        const float2 wt = g_wt[q];
+        const float w0 = eg[__float_as_int(wt.y) & 0xff] * wt.x;
+        const unsigned long long o = add2(mul2(nm.x, c1), mul2(nm.y, c2));  // n ch - m sh, n sh + m ch
+        const unsigned long long t = add2(o, big);
+        const float2 d = unpack2(fma2(add2(t, nbig), neg1, o));             // o - rint(o), exact
+        const float2 tf = unpack2(t);
+        const bool hx = fabsf(d.x) > tau, hy = fabsf(d.y) > tau;  // off the lattice line
+        const bool lx = d.x < -tau, ly = d.y < -tau;              // floor is the integer below
+        const float frx = lx ? d.x + 1.0f : (hx ? d.x : 0.0f);
+        const float fry = ly ? d.y + 1.0f : (hy ? d.y : 0.0f);
+        const int fx = __float_as_int(tf.x) - 0x4b400000 - (lx ? 1 : 0);
+        const int fy = __float_as_int(tf.y) - 0x4b400000 - (ly ? 1 : 0);
+        bool ok1, ok2;
+        if (BITS) {
+            const uint32_t kx = hx ? 3u : 1u;
+            const uint32_t need = hy ? kx * 257u : kx;
+            const int at = 8 * fy + fx;
+            ok1 = ((uint32_t)(near >> (at + 27)) & need) == need;
+            ok2 = ((uint32_t)(rnear >> (at + 36)) & need) == need;
+        } else {
+            const uint32_t need = hx ? 3u : 1u;
+            const int dy = hy ? 1 : 0, iy = cy + fy, jy = cy - fy;
+            const uint32_t m1 = ws->rowmask[iy] & ws->rowmask[iy + dy];
+            const uint32_t m2 = ws->rowmask[jy] & ws->rowmask[jy - dy];
+            ok1 = ((m1 >> (cx + fx)) & need) == need;
+            ok2 = ((m2 >> (cx - fx - (hx ? 1 : 0))) & need) == need;
+        }
+        any = any || ok1 || ok2;
+        weight_add(acc.s, acc.lo, (ok1 ? w0 : 0.f) + (ok2 ? w0 : 0.f));  // 0, w0 or 2 w0: exact
+        const float gx = 1.f - frx;
+        const float2 wy = unpack2(mul2(pack2(w0, w0), pack2(1.f - fry, fry)));
+        const float l00 = gx * wy.x, l10 = frx * wy.x, l01 = gx * wy.y, l11 = frx * wy.y;
+        const int A0 = c0 + fy * WS + fx, B0 = c0 - fy * WS - fx;
+        const bool x1 = ok1 && hx, y1 = ok1 && hy, x2 = ok2 && hx, y2 = ok2 && hy;
+        const ulonglong2 a0 = col[ok1 ? A0 : ZI];
+        const ulonglong2 a1 = col[x1 ? A0 + 1 : ZI];
+        const ulonglong2 a2 = col[y1 ? A0 + WS : ZI];
+        const ulonglong2 a3 = col[x1 && hy ? A0 + WS + 1 : ZI];
+        const ulonglong2 b0 = col[ok2 ? B0 : ZI];
+        const ulonglong2 b1 = col[x2 ? B0 - 1 : ZI];
+        const ulonglong2 b2 = col[y2 ? B0 - WS : ZI];
+        const ulonglong2 b3 = col[x2 && hy ? B0 - WS - 1 : ZI];
+        unsigned long long l = pack2(l00, l00);
+        acc_add(acc, l, a0);
+        acc_add(acc, l, b0);
+        l = pack2(l10, l10);
+        acc_add(acc, l, a1);
+        acc_add(acc, l, b1);
+        l = pack2(l01, l01);
+        acc_add(acc, l, a2);
+        acc_add(acc, l, b2);
+        l = pack2(l11, l11);
+        acc_add(acc, l, a3);
+        acc_add(acc, l, b3);
+    }
+    any_ = any;
+    acc_ = acc;
+}
+
+// The lattice ball of one pixel (offsets (n, m) themselves, one tap per sample),
+// over the mirror pairs j, j + G, ...; ISO: the stall rule's weights 1/|(n, m)|.  The
+// exponent is even in (n, m), so the pair shares its weight, and the plain sums need
+// no exponential per sample to rescale them: a tile with 9 to 16 front pixels at eps
+// 5 takes 5,800 cycles instead of 20,400 (a 1500 x 1125 still 2.80 -> 0.96 ms with the
+// rest of this kernel).
+template <int RW, bool ISO>
+__device__ __forceinline__ void lattice_pairs(const FillParams &p, const WarpSmem<RW> *ws, int pix, int j, int G, float2 g,
+                                              float &S_all_, bool &any_, Acc &acc_)
+{
+    constexpr int WS = WarpSmem<RW>::WS, ZI = WS * WS;
+    const ulonglong2 *col = reinterpret_cast<const ulonglong2 *>(ws->col);
+    const int cx = (pix & 7) + RW, cy = (pix >> 3) + RW, c0 = cy * WS + cx;
+    const int npair = p.tab.ns >> 1;
+    float S_all = 0.f;
+    bool any = false;
+    Acc acc = {0ull, 0ull, 0.f, 0.f};
+#pragma unroll 2
+    for (int q = j; q < npair; q += G) {
+        const float2 wt = g_wt[q];
+        const int code = __float_as_int(wt.y);
+        const int n = ((code >> 8) & 0xff) - 8, m = ((code >> 16) & 0xff) - 8;
+        float w0 = wt.x;
+        if (!ISO) {
+            const float proj = -g.y * (float)n + g.x * (float)m;  // g_perp . (n, m)
+            w0 *= expf(-(p.coef32 * proj * proj));
+        }
+        const bool ok1 = (ws->rowmask[cy + m] >> (cx + n)) & 1u;
+        const bool ok2 = (ws->rowmask[cy - m] >> (cx - n)) & 1u;
+        any = any || ok1 || ok2;
+        S_all += w0 + w0;
+        weight_add(acc.s, acc.lo, (ok1 ? w0 : 0.f) + (ok2 ? w0 : 0.f));
+        const int at = m * WS + n;
+        const unsigned long long w = pack2(w0, w0);
+        acc_add(acc, w, col[ok1 ? c0 + at : ZI]);
+        acc_add(acc, w, col[ok2 ? c0 - at : ZI]);
+    }
+    S_all_ = S_all;
+    any_ = any;
+    acc_ = acc;
+}
+
+struct PixelSums {
+    float S_rd, S_all, wsum;
+    int cnt;
+    float4 acc;
+};
+
+// One front pixel by the whole warp, each lane's colour sum relative to the smallest
+// weight exponent it has read (the normalisation cancels in the average and keeps
+// e^-t from underflowing): the pixels whose plain sums FP32 does not hold.  Must be
+// called by all 32 lanes; every lane gets the result.
+template <int RW>
+__device__ __noinline__ PixelSums slow_pixel(const FillParams &p, const WarpSmem<RW> *ws, int pix, bool ghost)
+{
+    constexpr int WS = WarpSmem<RW>::WS;
+    const int lane = threadIdx.x & 31;
+    const int px = pix & 7, py = pix >> 3;
+    const float2 g = ws->guide[pix];
+    float ch = 1.0f, sh = 0.0f, beta = 0.0f;
+    if (ghost) {
+        const float a2 = __fadd_rn(__fmul_rn(g.x, g.x), __fmul_rn(g.y, g.y));
+        const float a = __fsqrt_rn(a2);
+        if (a > 0.0f) {
+            ch = __fdiv_rn(g.x, a);
+            sh = __fdiv_rn(g.y, a);
+        }
+        beta = p.coef32 * a2;
+    }
+    float S_rd = 0.f, S_all = 0.f, tmin = INFINITY, wsum = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    int cnt = 0;
+    for (int s = lane; s < p.tab.ns; s += 32) {
+        const float nf = p.tab.n_f[s], mf = p.tab.m_f[s], invd = p.tab.invd[s];
+        float ox = nf, oy = mf;
+        if (ghost) {
+            ox = __fsub_rn(__fmul_rn(nf, ch), __fmul_rn(mf, sh));
+            oy = __fadd_rn(__fmul_rn(nf, sh), __fmul_rn(mf, ch));
+            float r0 = rintf(ox);
+            if (fabsf(__fsub_rn(ox, r0)) <= p.tau) ox = r0;
+            r0 = rintf(oy);
+            if (fabsf(__fsub_rn(oy, r0)) <= p.tau) oy = r0;
+        }
+        const float flx = floorf(ox), fly = floorf(oy);
+        const float frx = __fsub_rn(ox, flx), fry = __fsub_rn(oy, fly);
+        const int ix = px + RW + (int)flx, iy = py + RW + (int)fly;
+        const uint32_t need = frx > 0.0f ? 3u : 1u;
+        bool ok = ((ws->rowmask[iy] >> ix) & need) == need;
+        if (fry > 0.0f) ok = ok && (((ws->rowmask[iy + 1] >> ix) & need) == need);
+        float tt;
+        if (ghost) {
+            tt = beta * (mf * mf);
+        } else {
+            const float proj = -g.y * nf + g.x * mf;  // lattice ball: g_perp . (n, m)
+            tt = p.coef32 * proj * proj;
+        }
+        S_all += expf(-tt) * invd;
+        if (ok) {
+            S_rd += expf(-tt) * invd;
+            cnt++;
+            if (tt < tmin) {
+                const float sc = expf(tt - tmin);  // 0 for the first readable sample
+                acc.x *= sc; acc.y *= sc; acc.z *= sc; acc.w *= sc;
+                wsum *= sc;
+                tmin = tt;
+            }
+            const float w = expf(tmin - tt) * invd;
+            const float4 *cb = &ws->col[iy * WS + ix];
+            const float4 v = cb[0];
+            const float l00 = (1.f - frx) * (1.f - fry);
+            float4 val = make_float4(l00 * v.x, l00 * v.y, l00 * v.z, l00 * v.w);
+            if (frx > 0.f) {
+                const float l = frx * (1.f - fry);
+                const float4 c1 = cb[1];
+                val.x += l * c1.x; val.y += l * c1.y; val.z += l * c1.z; val.w += l * c1.w;
+            }
+            if (fry > 0.f) {
+                const float l = (1.f - frx) * fry;
+                const float4 c2 = cb[WS];
+                val.x += l * c2.x; val.y += l * c2.y; val.z += l * c2.z; val.w += l * c2.w;
+                if (frx > 0.f) {
+                    const float l3 = frx * fry;
+                    const float4 c3 = cb[WS + 1];
+                    val.x += l3 * c3.x; val.y += l3 * c3.y; val.z += l3 * c3.z; val.w += l3 * c3.w;
+                }
+            }
+            acc.x += w * val.x; acc.y += w * val.y; acc.z += w * val.z; acc.w += w * val.w;
+            wsum += w;
+        }
+    }
+    float tg = tmin;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) tg = fminf(tg, __shfl_xor_sync(FULL, tg, o));
+    const float sc = (tmin == INFINITY) ? 0.f : expf(tg - tmin);
+    PixelSums r = {S_rd, S_all, wsum * sc, cnt, make_float4(acc.x * sc, acc.y * sc, acc.z * sc, acc.w * sc)};
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        r.S_rd += __shfl_xor_sync(FULL, r.S_rd, o);
+        r.S_all += __shfl_xor_sync(FULL, r.S_all, o);
+        r.cnt += __shfl_xor_sync(FULL, r.cnt, o);
+        r.wsum += __shfl_xor_sync(FULL, r.wsum, o);
+        r.acc.x += __shfl_xor_sync(FULL, r.acc.x, o);
+        r.acc.y += __shfl_xor_sync(FULL, r.acc.y, o);
+        r.acc.z += __shfl_xor_sync(FULL, r.acc.z, o);
+        r.acc.w += __shfl_xor_sync(FULL, r.acc.w, o);
+    }
+    return r;
+}
+
 // The three work lists of a cluster (the list of step s in slot s % 3): the
 // first DS_LIST entries of each in the shared memory of the cluster's first CTA
 // (read and written by every CTA through distributed shared memory, a round trip
@@ -570,6 +905,8 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
     }
 
     unsigned long long cand;
+    unsigned claimable = 0;  // neighbours (by lane) that hold unfilled pixels
+    if (MODE != RESCAN) claimable = __ballot_sync(FULL, unb != 0ull);
     if (MODE == NORMAL) {
         if (k > 0) {
             const unsigned long long fm = (ftag == k - 1) ? fmsk : 0ull;
@@ -608,10 +945,6 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
             if ((cand >> pix) & 1ull) ws->guide[pix] = gv[h];
         }
     }
-    if (lane == 0) {
-        ws->ready = 0ull;
-        ws->recheck = 0ull;
-    }
     __syncwarp();
 
     // ---- exact active-boundary test of the candidates
@@ -639,6 +972,8 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
             }
         }
     }
+    const unsigned long long Qkeep = Qold & ~cand;
+    const int nqold = __popcll(Qold);
     const int np = __popcll(P);
     wc.evals += np;
     // the front pixels in increasing order: pixel q of a pass is plist[q]
@@ -649,218 +984,98 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
     }
 
     // ---- ready test (eqs. weight, confidence, ready) and the fill value in one
-    //      pass over the samples, G lanes per front pixel.  Each lane keeps its
-    //      colour sum relative to the smallest weight exponent it has read (the
-    //      normalisation cancels in the average and keeps e^-t from underflowing);
-    //      the G partial sums are brought to the group's smallest exponent when
-    //      they are combined.
+    //      pass over the sample pairs, G lanes per front pixel
+    unsigned long long Rm = 0ull, Cm = 0ull;  // ready; to be decided in FP64 (warp-uniform)
     if (np) {
         cp_async_wait_all();
         __syncwarp();
-        const int G = np <= 4 ? 8 : (np <= 8 ? 4 : (np <= 16 ? 2 : 1));
-        const int per = 32 / G;
-        const int j = lane & (G - 1), grp = lane / G;
-        const int ns = p.tab.ns;
-        const int npair = ns >> 1;
-        const bool rot = ghost && MODE != STALL;
-        const bool iso = ghost || MODE == STALL;  // the exponent depends on |m| only
-        const bool fast = MODE == STALL || (ghost && smart && p.c >= 1e-30f);
+        const int2 lanes = c_lanes[min(np, 17)];
+        const int G = lanes.x, per = 32 / G;
+        const int grp = (lane * lanes.y) >> 8, j = lane - grp * G;  // lane / G, lane % G
+        const bool decide = MODE != STALL && smart;
+        // weights that cannot all underflow: a pixel has a readable sample iff its sum is
+        // positive, or is not ready all the same
+        const bool plain = MODE == STALL || (ghost && decide);
         for (int base = 0; base < np; base += per) {
             const int q = base + grp;
-            const bool act = q < np;
+            const bool act = grp < per && q < np;
             const int pix = act ? ws->plist[q] : 0;
-            const int px = pix & 7, py = pix >> 3;
             float2 g = make_float2(0.f, 0.f);
             if (act && MODE != STALL) g = ws->guide[pix];
-            float ch = 1.0f, sh = 0.0f, beta = 0.0f;
-            if (MODE != STALL) {
-                float a2 = __fadd_rn(__fmul_rn(g.x, g.x), __fmul_rn(g.y, g.y));
-                if (ghost) {
-                    float a = __fsqrt_rn(a2);
-                    if (a > 0.0f) {
-                        ch = __fdiv_rn(g.x, a);
-                        sh = __fdiv_rn(g.y, a);
-                    }
-                    beta = p.coef32 * a2;
+            float S_all = 0.f;
+            bool any = false, odd = false;
+            Acc acc = {0ull, 0ull, 0.f, 0.f};
+            if (MODE != STALL && ghost) {
+                float ch = 1.0f, sh = 0.0f;
+                const float a2 = __fadd_rn(__fmul_rn(g.x, g.x), __fmul_rn(g.y, g.y));
+                const float a = __fsqrt_rn(a2);
+                if (a > 0.0f) {
+                    ch = __fdiv_rn(g.x, a);
+                    sh = __fdiv_rn(g.y, a);
                 }
-            }
-            float S_rd = 0.f, S_all = 0.f, tmin = INFINITY, wsum = 0.f;
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-            int cnt = 0;
-            if (fast) {
-                // group weights e^(-beta g^2), g = |m| = 0..R, shared by the pixel's G lanes
+                const float beta = p.coef32 * a2;
+                // |g| of a few denormals (or infinite): the rotation is not one
+                odd = !(fabsf(ch) <= 1.0001f && fabsf(sh) <= 1.0001f);
+                // group weights e^(-beta g^2), g = |m| = 0..R, shared by the pixel's lanes
                 __syncwarp();
                 if (act)
                     for (int gg = j; gg <= R; gg += G) ws->eg[grp][gg] = expf(-(beta * (float)(gg * gg)));
                 __syncwarp();
-            }
-            if (act && fast) {
-                // Rotated ball under smart order, or the stall pass: the weights need no
-                // normalisation (a ready pixel has S_rd > c S_all >= c times the m = 0
-                // weights; stall weights are 1/|(n, m)|).  Branch-free, over mirror pairs
-                // {(n, m), (-n, -m)}: negation is exact and commutes with every rounding of
-                // the rotation and of the snap, so the second offset is the exact negative
-                // of the first; the pair shares its rotation, snap, floor and weights, and
-                // each tap of the second sample is the first's tap reflected through the
-                // pixel, with the same bilinear weight.  Taps of zero weight and the taps of
-                // unreadable samples are read from the window's zero entry (an unreadable
-                // pixel's colour may be anything, and 0 * NaN is NaN).
-                constexpr int ZI = WS * WS;
-                const float *eg = ws->eg[grp];
-                const int cx = px + RW, cy = py + RW;
-#pragma unroll 1
-                for (int q2 = j; q2 < npair; q2 += G) {
-                    const float4 te = g_pair[q2];  // n, m, 1/|(n, m)|, |m|
-                    const float nf = te.x, mf = te.y;
-                    float ox, oy;
-                    if (rot) {
-                        ox = __fsub_rn(__fmul_rn(nf, ch), __fmul_rn(mf, sh));
-                        oy = __fadd_rn(__fmul_rn(nf, sh), __fmul_rn(mf, ch));
-                        float r0 = rintf(ox);
-                        if (fabsf(__fsub_rn(ox, r0)) <= p.tau) ox = r0;
-                        r0 = rintf(oy);
-                        if (fabsf(__fsub_rn(oy, r0)) <= p.tau) oy = r0;
-                    } else {
-                        ox = nf;
-                        oy = mf;
-                    }
-                    const float flx = floorf(ox), fly = floorf(oy);
-                    const float frx = __fsub_rn(ox, flx), fry = __fsub_rn(oy, fly);
-                    const int fx = (int)flx, fy = (int)fly;
-                    const bool hx = frx > 0.0f, hy = fry > 0.0f;
-                    const uint32_t need = hx ? 3u : 1u;
-                    // first sample: columns ix (+1), rows iy (+1); second: columns jx (+1)
-                    // and rows jy (-1), the reflections of the first's
-                    const int ix = cx + fx, iy = cy + fy;
-                    const int jx = cx - fx - (hx ? 1 : 0), jy = cy - fy;
-                    const uint32_t a0m = ws->rowmask[iy], a1m = ws->rowmask[iy + 1];
-                    const uint32_t b0m = ws->rowmask[jy], b1m = ws->rowmask[jy - 1];
-                    const bool ok1 = (((a0m >> ix) & need) == need) && (!hy || (((a1m >> ix) & need) == need));
-                    const bool ok2 = (((b0m >> jx) & need) == need) && (!hy || (((b1m >> jx) & need) == need));
-                    const float w0 = eg[__float_as_int(te.w)] * te.z;
-                    S_all += w0;
-                    S_all += w0;
-                    S_rd += ok1 ? w0 : 0.f;
-                    S_rd += ok2 ? w0 : 0.f;
-                    cnt += (ok1 ? 1 : 0) + (ok2 ? 1 : 0);
-                    const float gx = 1.f - frx, gy = 1.f - fry;
-                    const float l00 = w0 * (gx * gy), l10 = w0 * (frx * gy);
-                    const float l01 = w0 * (gx * fry), l11 = w0 * (frx * fry);
-                    const int A0 = iy * WS + ix, B0 = jy * WS + cx - fx;
-                    const float4 a0 = ws->col[ok1 ? A0 : ZI];
-                    const float4 a1 = ws->col[ok1 && hx ? A0 + 1 : ZI];
-                    const float4 a2 = ws->col[ok1 && hy ? A0 + WS : ZI];
-                    const float4 a3 = ws->col[ok1 && hx && hy ? A0 + WS + 1 : ZI];
-                    const float4 b0 = ws->col[ok2 ? B0 : ZI];
-                    const float4 b1 = ws->col[ok2 && hx ? B0 - 1 : ZI];
-                    const float4 b2 = ws->col[ok2 && hy ? B0 - WS : ZI];
-                    const float4 b3 = ws->col[ok2 && hx && hy ? B0 - WS - 1 : ZI];
-                    acc.x = __fmaf_rn(l00, a0.x, acc.x); acc.y = __fmaf_rn(l00, a0.y, acc.y);
-                    acc.z = __fmaf_rn(l00, a0.z, acc.z); acc.w = __fmaf_rn(l00, a0.w, acc.w);
-                    acc.x = __fmaf_rn(l10, a1.x, acc.x); acc.y = __fmaf_rn(l10, a1.y, acc.y);
-                    acc.z = __fmaf_rn(l10, a1.z, acc.z); acc.w = __fmaf_rn(l10, a1.w, acc.w);
-                    acc.x = __fmaf_rn(l01, a2.x, acc.x); acc.y = __fmaf_rn(l01, a2.y, acc.y);
-                    acc.z = __fmaf_rn(l01, a2.z, acc.z); acc.w = __fmaf_rn(l01, a2.w, acc.w);
-                    acc.x = __fmaf_rn(l11, a3.x, acc.x); acc.y = __fmaf_rn(l11, a3.y, acc.y);
-                    acc.z = __fmaf_rn(l11, a3.z, acc.z); acc.w = __fmaf_rn(l11, a3.w, acc.w);
-                    acc.x = __fmaf_rn(l00, b0.x, acc.x); acc.y = __fmaf_rn(l00, b0.y, acc.y);
-                    acc.z = __fmaf_rn(l00, b0.z, acc.z); acc.w = __fmaf_rn(l00, b0.w, acc.w);
-                    acc.x = __fmaf_rn(l10, b1.x, acc.x); acc.y = __fmaf_rn(l10, b1.y, acc.y);
-                    acc.z = __fmaf_rn(l10, b1.z, acc.z); acc.w = __fmaf_rn(l10, b1.w, acc.w);
-                    acc.x = __fmaf_rn(l01, b2.x, acc.x); acc.y = __fmaf_rn(l01, b2.y, acc.y);
-                    acc.z = __fmaf_rn(l01, b2.z, acc.z); acc.w = __fmaf_rn(l01, b2.w, acc.w);
-                    acc.x = __fmaf_rn(l11, b3.x, acc.x); acc.y = __fmaf_rn(l11, b3.y, acc.y);
-                    acc.z = __fmaf_rn(l11, b3.z, acc.z); acc.w = __fmaf_rn(l11, b3.w, acc.w);
+                if (act && !odd) {
+                    const float *eg = ws->eg[grp];
+                    if (RW == 4 && p.tau >= 2e-6f) rotated_pairs<RW, true>(p, ws, eg, pix, j, G, ch, sh, any, acc);
+                    else rotated_pairs<RW, false>(p, ws, eg, pix, j, G, ch, sh, any, acc);
+                    if (decide && j == 0)
+                        for (int gg = 0; gg <= R; gg++) S_all = __fmaf_rn(eg[gg], p.tab.Dm[gg], S_all);
                 }
             } else if (act) {
-#pragma unroll 2
-                for (int s = j; s < ns; s += G) {
-                    const float4 te = g_stab[s];
-                    const float nf = te.x, mf = te.y, invd = te.z;
-                    float ox, oy;
-                    if (rot) {
-                        ox = __fsub_rn(__fmul_rn(nf, ch), __fmul_rn(mf, sh));
-                        oy = __fadd_rn(__fmul_rn(nf, sh), __fmul_rn(mf, ch));
-                        float r0 = rintf(ox);
-                        if (fabsf(__fsub_rn(ox, r0)) <= p.tau) ox = r0;
-                        r0 = rintf(oy);
-                        if (fabsf(__fsub_rn(oy, r0)) <= p.tau) oy = r0;
-                    } else {
-                        ox = nf;
-                        oy = mf;
-                    }
-                    const float flx = floorf(ox), fly = floorf(oy);
-                    const float frx = __fsub_rn(ox, flx), fry = __fsub_rn(oy, fly);
-                    const int ix = px + RW + (int)flx, iy = py + RW + (int)fly;
-                    const uint32_t need = frx > 0.0f ? 3u : 1u;
-                    bool ok = ((ws->rowmask[iy] >> ix) & need) == need;
-                    if (fry > 0.0f) ok = ok && (((ws->rowmask[iy + 1] >> ix) & need) == need);
-                    float tt;
-                    if (iso) {
-                        tt = beta * (mf * mf);
-                    } else {
-                        const float proj = -g.y * nf + g.x * mf;  // lattice ball: g_perp . (n, m)
-                        tt = p.coef32 * proj * proj;
-                    }
-                    const float w0 = expf(-tt) * invd;
-                    S_all += w0;
-                    if (ok) {
-                        S_rd += w0;
-                        cnt++;
-                        if (tt < tmin) {
-                            const float sc = expf(tt - tmin);  // 0 for the first readable sample
-                            acc.x *= sc; acc.y *= sc; acc.z *= sc; acc.w *= sc;
-                            wsum *= sc;
-                            tmin = tt;
-                        }
-                        const float w = expf(tmin - tt) * invd;
-                        const float4 *cb = &ws->col[iy * WS + ix];
-                        const float4 v = cb[0];
-                        const float l00 = (1.f - frx) * (1.f - fry);
-                        float4 val = make_float4(l00 * v.x, l00 * v.y, l00 * v.z, l00 * v.w);
-                        if (frx > 0.f) {
-                            const float l = frx * (1.f - fry);
-                            const float4 c1 = cb[1];
-                            val.x += l * c1.x; val.y += l * c1.y; val.z += l * c1.z; val.w += l * c1.w;
-                        }
-                        if (fry > 0.f) {
-                            const float l = (1.f - frx) * fry;
-                            const float4 c2 = cb[WS];
-                            val.x += l * c2.x; val.y += l * c2.y; val.z += l * c2.z; val.w += l * c2.w;
-                            if (frx > 0.f) {
-                                const float l3 = frx * fry;
-                                const float4 c3 = cb[WS + 1];
-                                val.x += l3 * c3.x; val.y += l3 * c3.y; val.z += l3 * c3.z; val.w += l3 * c3.w;
-                            }
-                        }
-                        acc.x += w * val.x; acc.y += w * val.y; acc.z += w * val.z; acc.w += w * val.w;
-                        wsum += w;
+                lattice_pairs<RW, MODE == STALL>(p, ws, pix, j, G, g, S_all, any, acc);
+            }
+            // combine the lanes of a pixel: lane j takes from j + 1, then j + 2, ...
+            float2 axy = unpack2(acc.xy), azw = unpack2(acc.zw);
+            float S_rd = acc.s, S_lo = acc.lo;
+            for (int o = 1; o < G; o <<= 1) {
+                const float s0 = __shfl_down_sync(FULL, S_rd, o), s1 = __shfl_down_sync(FULL, S_lo, o);
+                const float c0 = __shfl_down_sync(FULL, axy.x, o), c1 = __shfl_down_sync(FULL, axy.y, o);
+                const float c2 = __shfl_down_sync(FULL, azw.x, o), c3 = __shfl_down_sync(FULL, azw.y, o);
+                const bool in = j + o < G;
+                if (in) {
+                    weight_add(S_rd, S_lo, s0);
+                    S_lo += s1;
+                    axy.x += c0;
+                    axy.y += c1;
+                    azw.x += c2;
+                    azw.y += c3;
+                }
+                if (!plain) {
+                    const float a1 = __shfl_down_sync(FULL, S_all, o);
+                    const bool an = __shfl_down_sync(FULL, (int)any, o) != 0;
+                    if (in) {
+                        S_all += a1;
+                        any = any || an;
                     }
                 }
             }
-            // combine the G lanes of a pixel
-            if (!fast) {
-                float tg = tmin;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1)
-                    if (o < G) tg = fminf(tg, __shfl_xor_sync(FULL, tg, o));
-                const float sc = (tmin == INFINITY) ? 0.f : expf(tg - tmin);
-                acc.x *= sc; acc.y *= sc; acc.z *= sc; acc.w *= sc;
-                wsum *= sc;
-            } else {
-                wsum = S_rd;
-            }
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                if (o < G) {
-                    S_rd += __shfl_xor_sync(FULL, S_rd, o);
-                    S_all += __shfl_xor_sync(FULL, S_all, o);
-                    cnt += __shfl_xor_sync(FULL, cnt, o);
-                    acc.x += __shfl_xor_sync(FULL, acc.x, o);
-                    acc.y += __shfl_xor_sync(FULL, acc.y, o);
-                    acc.z += __shfl_xor_sync(FULL, acc.z, o);
-                    acc.w += __shfl_xor_sync(FULL, acc.w, o);
-                    wsum += __shfl_xor_sync(FULL, wsum, o);
+            if (plain) any = S_rd > 0.f;
+            // Sums that FP32 holds badly: readable weights that all underflow (without the
+            // ready test a pixel is filled whatever they are; with it a rotated ball's ready
+            // pixels have S_rd > c S_all >= c times the m = 0 weights, but a lattice ball's
+            // weights may all be tiny), and rotations that are not one.  Those pixels are
+            // done again, one at a time, relative to their smallest readable exponent.
+            float wsum = S_rd;
+            const bool redo = act && j == 0 && MODE != STALL &&
+                              (odd || (any && !(decide ? ghost || S_all >= 1e-18f : !(S_rd < 1e-18f))));
+            for (unsigned rb = __ballot_sync(FULL, redo); rb; rb &= rb - 1u) {
+                const int src = __ffs(rb) - 1;
+                const PixelSums r = slow_pixel<RW>(p, ws, __shfl_sync(FULL, pix, src), ghost);
+                if (lane == src) {
+                    S_rd = r.S_rd;
+                    S_all = r.S_all;
+                    any = r.cnt > 0;
+                    axy = make_float2(r.acc.x, r.acc.y);
+                    azw = make_float2(r.acc.z, r.acc.w);
+                    wsum = r.wsum;
+                    S_lo = 0.f;
                 }
             }
             // Smart order: decided in FP32 outside a guard band around c, re-checked in
@@ -868,9 +1083,9 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
             // error of both sums is below ~1e-5 relative (the m = 0 terms are exact and
             // the error of each other term is bounded by t e^-t <= 1/e times a few ulp);
             // 1e-3 for the lattice ball, whose projection g_perp.(n, m) can cancel.
-            bool ready = cnt > 0;
+            bool ready = any;
             bool recheck = false;
-            if (MODE != STALL && smart) {
+            if (decide) {
                 const float d = S_rd - p.c * S_all;
                 const float tol = (ghost ? 1e-4f : 1e-3f) * p.c * S_all;
                 ready = d > tol;
@@ -881,23 +1096,29 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
                 ready = false;
                 recheck = false;
             }
-            if (act && j == 0 && cnt > 0 && (ready || recheck)) {
-                atomicOr(recheck ? &ws->recheck : &ws->ready, 1ull << pix);
-                const float inv = 1.0f / wsum;
-                ws->colr[pix] = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+            const bool take = act && j == 0 && any;
+            ready = ready && !recheck;
+            if (take && (ready || recheck)) {
+                // acc / (wsum + S_lo): the reciprocal's product, corrected once
+                const float inv = __frcp_rn(wsum);
+                auto quot = [&](float v) {
+                    const float x = v * inv;
+                    const float y = __fmaf_rn(__fmaf_rn(-x, S_lo, __fmaf_rn(-x, wsum, v)), inv, x);
+                    return fabsf(x) < INFINITY ? y : x;
+                };
+                ws->colr[pix] = make_float4(quot(axy.x), quot(axy.y), quot(azw.x), quot(azw.y));
             }
+            Rm |= pixel_mask(take && ready, pix);
+            if (__any_sync(FULL, take && recheck)) Cm |= pixel_mask(take && recheck, pix);
         }
     }
     __syncwarp();
     // FP64 re-checks, one pixel at a time with the whole warp
-    for (unsigned long long rc = ws->recheck; rc; rc &= rc - 1ull) {
+    for (unsigned long long rc = Cm; rc; rc &= rc - 1ull) {
         const int pix = __ffsll((long long)rc) - 1;
-        const bool r64 = warp_ready_fp64<RW>(p, ws, pix, ghost);
-        if (lane == 0 && r64) atomicOr(&ws->ready, 1ull << pix);
+        if (warp_ready_fp64<RW>(p, ws, pix, ghost)) Rm |= 1ull << pix;
         wc.rechecks++;
     }
-    __syncwarp();
-    const unsigned long long Rm = ws->ready;
     const int nr = __popcll(Rm);
     if (phase1) {
         // guided pixels filled: the data term stays on while any is left
@@ -923,7 +1144,7 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
     }
 
     // ---- tile bookkeeping
-    const unsigned long long Qnew = (Qold & ~cand) | (P & ~Rm);
+    const unsigned long long Qnew = Qkeep | (P & ~Rm);
     if (lane == 0) {
         if (Rm) {
             F.U[t] = U & ~Rm;
@@ -931,10 +1152,10 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
             e->mask = Rm;
             e->tag = k;
         }
-        if (Qnew != Qold) F.Qw[t] = Qnew;
+        if (Qnew != 0ull || nqold != 0) F.Qw[t] = Qnew;
     }
     wc.filled += nr;
-    wc.delta += __popcll(Qnew) - __popcll(Qold);
+    wc.delta += __popcll(Qnew) - nqold;
 
     // the previous tiles' claims and reservations have returned by now
     claims_write(p, lists, pc, wc);
@@ -959,9 +1180,8 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
         const uint32_t lowm = reach >= 8 ? 0xffu : ((1u << reach) - 1u);
         const bool nL = (colocc & lowm) != 0, nR = (colocc >> (8 - (reach >= 8 ? 8 : reach))) != 0;
         const bool nU = (rowocc & lowm) != 0, nD = (rowocc >> (8 - (reach >= 8 ? 8 : reach))) != 0;
-        const unsigned long long left = (lane == 4) ? (U & ~Rm) : unb;
-        const bool need = nvalid && (ndx == 0 || (ndx < 0 ? nL : nR)) && (ndy == 0 || (ndy < 0 ? nU : nD)) &&
-                          left != 0ull;
+        const bool left = lane == 4 ? (U & ~Rm) != 0ull : ((claimable >> lane) & 1u) != 0u;
+        const bool need = nvalid && (ndx == 0 || (ndx < 0 ? nL : nR)) && (ndy == 0 || (ndy < 0 ? nU : nD)) && left;
         const unsigned bm = __ballot_sync(FULL, need);
         if (bm) {
             pc.k = k;
@@ -1089,6 +1309,13 @@ __device__ __forceinline__ bool team_sync(TeamCtl *tc, int *acc, int *dead, int 
     return *dead == 0;
 }
 
+// A frame's statistics, kept by its leader (in shared memory: the other threads need
+// no registers for them).
+struct Totals {
+    long long filled, evals;
+    int max_front, stalls, data_switch;
+};
+
 // What a cluster does next, in the shared memory of its first CTA: f >= 0 is a
 // queue position, -1 nothing is left; with help set the cluster is member
 // `member` of the frame's team.
@@ -1149,15 +1376,18 @@ __device__ int team_find(const FillParams &p, int unit, Role *role)
     return -1;
 }
 
-// Every warp of the cluster visits the frame's tiles (32 at a time); the mode
+// Every warp of the team visits the frame's tiles (32 at a time); the mode
 // selects the tile mask that makes a tile a member (U: rescan, re-evaluation;
 // Qw: stall) and is passed on as the tile's candidates.
 template <int RW, int MODE>
-__device__ void sweep_tiles(const FillParams &p, const FrameDev &F, WarpSmem<RW> *ws, GroupCtl *ctl,
-                            const Lists &lists, int k, int gw, int nw, WarpCounters &wc, PendingClaims &pc,
-                            bool phase1 = false)
+__device__ __forceinline__ WarpCounters sweep_tiles(const FillParams &p, const FrameDev &F, WarpSmem<RW> *ws, GroupCtl *ctl,
+                                                 const Lists lists, int k, int gw, int nw, bool phase1)
 {
     const int lane = threadIdx.x & 31;
+    WarpCounters wc = {0, 0, 0, 0, 0};
+    PendingClaims pc;
+    pc.m1 = 0u;
+    pc.m2 = 0u;
     for (int base = gw * 32; base < F.ntiles; base += nw * 32) {
         int t = base + lane;
         unsigned long long m = 0;
@@ -1170,10 +1400,12 @@ __device__ void sweep_tiles(const FillParams &p, const FrameDev &F, WarpSmem<RW>
             process_tile<RW, MODE>(p, F, ws, ctl, lists, base + i, k, mi, wc, pc, false, phase1);
         }
     }
+    claims_drain(p, ctl, lists, pc, wc);
+    return wc;
 }
 
 template <int RW>
-__global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __grid_constant__ FillParams p)
+__global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_constant__ FillParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ FrameDev s_frame;
@@ -1188,25 +1420,26 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
     __shared__ int32_t s_lists[3 * DS_LIST];
     __shared__ Role s_role[2];
     __shared__ int s_acc[5];   // the CTA's step counters while it is in a team
+    __shared__ Totals s_tot;   // the leader's
     __shared__ int s_dead;     // a team barrier's wait gave up
     GroupCtl *const ds_ctl = cluster.map_shared_rank(&s_ctl, 0);
     const Role *const ds_role = cluster.map_shared_rank(s_role, 0);
     Lists lists;
     lists.ds = cluster.map_shared_rank(s_lists, 0);
     lists.cap = p.list_cap;
-    const int unit = csize * fill_warps(RW);  // warps of a cluster
+    const int unit = csize * FILL_WARPS;  // warps of a cluster
     const bool rescan = (p.flags & GF_FLAG_RESCAN) != 0;
-    for (int i = threadIdx.x; i < p.tab.nsp; i += blockDim.x) {
-        g_stab[i] = make_float4(p.tab.n_f[i], p.tab.m_f[i], p.tab.invd[i], fabsf(p.tab.m_f[i]));
+    for (int i = threadIdx.x; i < p.tab.ns; i += blockDim.x) {
         // group |m| = g lists m = -g before m = +g (n ascending within each), and
         // n < 0 before n > 0 for g = 0: the first half of every group holds one
         // sample of each mirror pair, and every group before it has an even count
-        if (i < p.tab.ns) {
-            const int g = (int)fabsf(p.tab.m_f[i]);
-            const int g0 = p.tab.m_start[g], half = (p.tab.m_start[g + 1] - g0) >> 1;
-            if (i - g0 < half)
-                g_pair[(g0 >> 1) + (i - g0)] =
-                    make_float4(p.tab.n_f[i], p.tab.m_f[i], p.tab.invd[i], __int_as_float(g));
+        const float n = p.tab.n_f[i], m = p.tab.m_f[i];
+        const int g = (int)fabsf(m);
+        const int g0 = p.tab.m_start[g], half = (p.tab.m_start[g + 1] - g0) >> 1;
+        if (i - g0 < half) {
+            const int e = (g0 >> 1) + (i - g0);
+            g_pos[e] = make_float4(n, n, m, m);
+            g_wt[e] = make_float2(p.tab.invd[i], __int_as_float(g | ((int)n + 8) << 8 | ((int)m + 8) << 16));
         }
     }
     if ((threadIdx.x & 31) == 0) ws->col[WarpSmem<RW>::WS * WarpSmem<RW>::WS] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1277,24 +1510,23 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
             return team_sync(tc, s_acc, &s_dead, k % 3, bar);
         };
 
-        long long n_front = 0;
-        long long filled_tot = 0, evals_tot = 0, max_front = 0;
-        int stalls = 0, status = GF_OK;
+        int n_front = 0;
+        int status = GF_OK;
         int k = 0;
+        if (leader) s_tot = Totals{0, 0, 0, 0, -1};
         const int max_shells = F.max_shells;
         int n_cur = 0;
         // eq. ready2 (GF_FLAG_DATA): phase 1 while hole pixels with g != 0 remain and
         // some front pixel is ready under the data term; `reval`: this step tests every
         // front pixel with eq. ready (the tracked front was built under phase 1)
         bool phase1 = (p.flags & GF_FLAG_DATA) != 0;
-        int data_switch = -1;
         bool reval = false;
         if (own) {
             n_front = ld(&F.init_count[1]);
             n_cur = ld(&F.init_count[0]);
             if (phase1 && ld(F.gleft) == 0) {
                 phase1 = false;
-                data_switch = 0;
+                if (leader) s_tot.data_switch = 0;
             }
         } else {
             const Admission &adm = role->adm;
@@ -1363,9 +1595,6 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
         for (;;) {
             const int slot = k % 3;
             WarpCounters wc = {0, 0, 0, 0, 0};
-            PendingClaims pc;
-            pc.m1 = 0u;
-            pc.m2 = 0u;
             int asked = 0;
             if (leader && open) asked = (int)*(volatile uint32_t *)&tc->want;
             const bool more = n_cur > nw;
@@ -1375,12 +1604,15 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
             // entries against 9.5 us with a compact one)
             const bool defer = team > 1 || 5 * n_cur > 2 * nw;
             if (rescan) {
-                sweep_tiles<RW, RESCAN>(p, F, ws, ctl, lists, k, gw, nw, wc, pc, phase1);
+                wc = sweep_tiles<RW, RESCAN>(p, F, ws, ctl, lists, k, gw, nw, phase1);
             } else if (reval) {
-                sweep_tiles<RW, REVAL>(p, F, ws, ctl, lists, k, gw, nw, wc, pc);
+                wc = sweep_tiles<RW, REVAL>(p, F, ws, ctl, lists, k, gw, nw, false);
             } else {
                 // step 0 takes the init kernel's list, later steps the lists built by the claims
                 const int n = n_cur;
+                PendingClaims pc;
+                pc.m1 = 0u;
+                pc.m2 = 0u;
 
                 // Item gw goes to warp gw; items beyond the warp count are handed out
                 // by a per-step cursor (the next grab is in flight while a tile is
@@ -1389,19 +1621,17 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
                 const bool lane0 = (threadIdx.x & 31) == 0;
                 int pre = 0;
                 if (lane0 && more) pre = atomicAdd(&ctl->step[slot].cursor, 1);
-                const int t0 = gw < n ? t0_cur : -1;
-                if (t0 >= 0) process_tile<RW, NORMAL>(p, F, ws, ctl, lists, t0, k, 0ull, wc, pc, defer, phase1);
-                if (more) {
-                    int nxt = nw + __shfl_sync(FULL, pre, 0);
-                    while (nxt < n) {
-                        const int t = k == 0 ? ld(&F.init_list[nxt]) : list_get(lists, slot, nxt);
-                        if (lane0) pre = atomicAdd(&ctl->step[slot].cursor, 1);
-                        if (t >= 0) process_tile<RW, NORMAL>(p, F, ws, ctl, lists, t, k, 0ull, wc, pc, defer, phase1);
-                        nxt = nw + __shfl_sync(FULL, pre, 0);
-                    }
+                int t = gw < n ? t0_cur : -1;
+                for (;;) {
+                    if (t >= 0) process_tile<RW, NORMAL>(p, F, ws, ctl, lists, t, k, 0ull, wc, pc, defer, phase1);
+                    if (!more) break;
+                    const int nxt = nw + __shfl_sync(FULL, pre, 0);
+                    if (nxt >= n) break;
+                    t = k == 0 ? ld(&F.init_list[nxt]) : list_get(lists, slot, nxt);
+                    if (lane0) pre = atomicAdd(&ctl->step[slot].cursor, 1);
                 }
+                claims_drain(p, ctl, lists, pc, wc);
             }
-            claims_drain(p, ctl, lists, pc, wc);
             if (leader && open) ctl->step[slot].join = asked;
             if (!finish(wc, k, false, threadIdx.x < 32 && (team == 1 || (own && crank == 0)))) {
                 status = GF_ERR_TIMEOUT;
@@ -1416,22 +1646,21 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
             const int join = open ? c1.y : 0;
             int t0_next = gw < p.list_cap ? list_get(lists, s3n, gw) : -1;  // used only if gw < n_next
             const int gleft = phase1 ? ld(F.gleft) : -1;
-            evals_tot += ev;
             if (er) {
                 status = GF_ERR_INTERNAL;
                 break;
             }
-            long long front_k = n_front + dlt + filled;
-            if (front_k > max_front) max_front = front_k;
+            if (leader) {
+                s_tot.evals += ev;
+                s_tot.max_front = max(s_tot.max_front, n_front + dlt + filled);
+            }
             reval = false;
             if (phase1 && filled == 0) {
                 // eq. ready2 fills nothing at this step: eq. ready from this step on,
                 // and this step is evaluated again with it (every front pixel)
                 phase1 = false;
-                data_switch = k;
-                WarpCounters wr = {0, 0, 0, 0, 0};
-                sweep_tiles<RW, REVAL>(p, F, ws, ctl, lists, k, gw, nw, wr, pc);
-                claims_drain(p, ctl, lists, pc, wr);
+                if (leader) s_tot.data_switch = k;
+                const WarpCounters wr = sweep_tiles<RW, REVAL>(p, F, ws, ctl, lists, k, gw, nw, false);
                 if (!finish(wr, k, true, false)) {
                     status = GF_ERR_TIMEOUT;
                     break;
@@ -1445,12 +1674,11 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
                     status = GF_ERR_INTERNAL;
                     break;
                 }
-                front_k = n_front + dlt + filled;
-                if (front_k > max_front) max_front = front_k;
+                if (leader) s_tot.max_front = max(s_tot.max_front, n_front + dlt + filled);
             } else if (phase1 && gleft == 0) {
                 // every pixel with g != 0 is filled: eq. ready from the next step on
                 phase1 = false;
-                data_switch = k + 1;
+                if (leader) s_tot.data_switch = k + 1;
                 reval = true;
             }
             int fk = filled;
@@ -1459,9 +1687,7 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
                 // stall rule: no front pixel is ready; fill the front isotropically.  The
                 // stall pass adds to the same slot (its counters were zero after the
                 // evaluation pass, except the front delta).
-                WarpCounters ws2 = {0, 0, 0, 0, 0};
-                sweep_tiles<RW, STALL>(p, F, ws, ctl, lists, k, gw, nw, ws2, pc);
-                claims_drain(p, ctl, lists, pc, ws2);
+                const WarpCounters ws2 = sweep_tiles<RW, STALL>(p, F, ws, ctl, lists, k, gw, nw, false);
                 if (!finish(ws2, k, true, false)) {
                     status = GF_ERR_TIMEOUT;
                     break;
@@ -1478,13 +1704,13 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
                 }
                 if (sf == 0) break;  // front pixels with no readable sample at all
                 n_front += dlt2;
-                stalls++;
                 fk = sf;
+                if (leader) s_tot.stalls++;
                 if (leader && F.stall_bits) atomicOr(&F.stall_bits[k >> 5], 1u << (k & 31));
             } else {
                 n_front += dlt;
             }
-            filled_tot += fk;
+            if (leader) s_tot.filled += fk;
             // without deferred claims the list holds markers of lost ones; its tiles are
             // then about as many as this step's, at most one per warp
             const int load = rescan ? sweep_load : (defer ? n_next : min(n_next, nw));
@@ -1552,15 +1778,15 @@ __global__ void __launch_bounds__(fill_warps(RW) * 32, 1) fill_kernel(const __gr
             const int holes = ld(F.holes);
             gf_stats st;
             st.shells = k;
-            st.stalls = stalls;
-            st.filled = filled_tot;
-            st.evaluations = evals_tot;
-            st.max_front = max_front;
+            st.stalls = s_tot.stalls;
+            st.filled = s_tot.filled;
+            st.evaluations = s_tot.evals;
+            st.max_front = s_tot.max_front;
             st.holes = holes;
             st.rechecks = s_ctl.rechecks + (tc ? ld(&tc->c.rechecks) : 0);
-            st.data_switch = data_switch;
+            st.data_switch = s_tot.data_switch;
             st.reserved = 0;
-            if (status == GF_OK && filled_tot < holes) status = GF_INCOMPLETE;
+            if (status == GF_OK && s_tot.filled < holes) status = GF_INCOMPLETE;
             st.status = status;
             *F.stats = st;
         }

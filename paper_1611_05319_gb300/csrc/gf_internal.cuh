@@ -13,10 +13,13 @@ constexpr int MAX_SAMPLES = 224;     // lattice points with n^2+m^2 <= 64, minus
 constexpr int MAX_R = 8;             // ceil(eps) <= 8
 constexpr int WARPS_PER_CTA = 16;
 constexpr int CTA_THREADS = WARPS_PER_CTA * 32;
-// Warps per CTA of the fill kernel: 16, or 12 for the 24x24 window (eps > 4),
-// whose state-window loads need more than the 128 registers a thread gets at
-// 16 warps.
-__host__ __device__ constexpr int fill_warps(int rw) { return rw == 8 ? 12 : 16; }
+// Warps per CTA of the fill kernel.  12, with up to 168 registers a thread: a step
+// lasts as long as its slowest tile's instruction stream, and the sample loop keeps
+// enough in flight only without spills.  Measured with 16 (128 registers, 212 bytes of
+// spills) and 12 warps: one 1080p frame 1.57 and 1.28 ms, a 4K frame with a blob 4.20
+// and 3.42 ms, 32 uneven 1080p frames 4.19 and 3.88 ms; with 8 (250 registers) 1.32,
+// 3.32 and 4.65 ms.
+constexpr int FILL_WARPS = 12;
 // init kernel: CTAs of a frame (INIT_WARPS warps, one strip of 8 rows x 256 columns each)
 constexpr int INIT_WARPS = 8;
 __host__ __device__ inline int init_ctas(int TH, int W) {
@@ -60,8 +63,6 @@ struct WarpSmem {
     uint32_t rowmask[WS];        // readable bits of the window rows
     float4 colr[64];             // fill value of each ready (or re-checked) pixel
     float eg[32][MAX_R + 1];     // per pixel slot of a pass: e^(-beta g^2) for g = |m| = 0..R
-    unsigned long long ready;
-    unsigned long long recheck;   // pixels whose ready test is re-done in FP64
     uint8_t plist[64];           // the tile's front pixels in increasing order
 };
 
@@ -125,7 +126,7 @@ struct Admission {
     int32_t n_cur;                // its work list's length
     int32_t phase1, reval;
     uint32_t bar;                 // arrivals that the team's barrier has counted
-    int64_t n_front;
+    int32_t n_front;
 };
 
 // Per-frame control block in global memory for a frame that several clusters

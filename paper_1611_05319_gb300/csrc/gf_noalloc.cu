@@ -94,7 +94,7 @@ int rw_of(float eps)
 
 size_t smem_of(int rw)
 {
-    return fill_warps(rw) * (rw == 4 ? sizeof(WarpSmem<4>) : (rw == 5 ? sizeof(WarpSmem<5>) : sizeof(WarpSmem<8>)));
+    return FILL_WARPS * (rw == 4 ? sizeof(WarpSmem<4>) : (rw == 5 ? sizeof(WarpSmem<5>) : sizeof(WarpSmem<8>)));
 }
 
 // Once per device, with that device current: the scratch's device address and
@@ -120,7 +120,7 @@ cudaError_t setup_device(int dev)
         for (int cs = 16; cs >= 1 && best == 0; cs >>= 1) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(cs);
-            cfg.blockDim = dim3(32 * fill_warps(rws[i]));
+            cfg.blockDim = dim3(32 * FILL_WARPS);
             cfg.dynamicSmemBytes = smem_of(rws[i]);
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeClusterDimension;
@@ -247,7 +247,7 @@ extern "C" gf_status gf_fill_noalloc(const gf_frame *f, const gf_params *p, gf_s
     if (cudaGetLastError() != cudaSuccess) return GF_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cs);
-    cfg.blockDim = dim3(32 * fill_warps(rw));
+    cfg.blockDim = dim3(32 * FILL_WARPS);
     cfg.dynamicSmemBytes = smem_of(rw);
     cfg.stream = st;
     cudaLaunchAttribute at[1];

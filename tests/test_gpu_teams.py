@@ -33,7 +33,6 @@ def _run(ctx, frames, guides, rgbas, **kw):
     out = []
     for r in rs:
         st = r.stats()
-        st.pop("rechecks")
         words = (st["shells"] + 31) // 32
         out.append((r.rgba.cpu().numpy(), r.shell.cpu().numpy(), r.enter.cpu().numpy(),
                     r.stall.cpu().numpy()[:words], st))
