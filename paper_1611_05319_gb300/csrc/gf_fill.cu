@@ -354,7 +354,8 @@ __device__ bool warp_ready_fp64(const FillParams &p, const WarpSmem<RW> *ws, int
             const float frx = __fsub_rn(ox, flx), fry = __fsub_rn(oy, fly);
             const int ix = px + RW + (int)flx, iy = py + RW + (int)fly;
             const uint32_t need = frx > 0.0f ? 3u : 1u;
-            bool rd = ((ws->rowmask[iy] >> ix) & need) == need;
+            bool rd = ix >= 0 && iy >= 0 && ix < WarpSmem<RW>::WS - 1 && iy < WarpSmem<RW>::WS - 1;
+            rd = rd && ((ws->rowmask[iy] >> ix) & need) == need;
             if (fry > 0.0f) rd = rd && (((ws->rowmask[iy + 1] >> ix) & need) == need);
             double t;
             if (ghost) {
@@ -484,7 +485,8 @@ __device__ __forceinline__ unsigned long long around(const WarpSmem<RW> *ws, int
 // its sign) instead of the conversion unit; BITS: the readability of a sample's
 // cell as one shift and one mask of a register word, the mirrored sample's with the
 // same shift and mask of the reversed word, instead of four shared loads.  BITS
-// needs R <= 3 and a snap that covers the rotation's rounding, |offset| <= R.
+// needs R <= 3 and |offset| <= R after the snap: offsets exceed R by their rounding, at
+// most R (2.4e-7 + 2^-22) < 1.5e-6, so a snap of 6e-6 px and more covers it.
 // Measured (cycles of a tile's sample passes, one 1080p frame, eps 3): 9 to 16 front
 // pixels 8,200 -> 6,100, 17 and more 13,100 -> 8,900, an iteration 620 -> 450.
 template <int RW, bool BITS>
@@ -656,7 +658,9 @@ __device__ __noinline__ PixelSums slow_pixel(const FillParams &p, const WarpSmem
         const float frx = __fsub_rn(ox, flx), fry = __fsub_rn(oy, fly);
         const int ix = px + RW + (int)flx, iy = py + RW + (int)fly;
         const uint32_t need = frx > 0.0f ? 3u : 1u;
-        bool ok = ((ws->rowmask[iy] >> ix) & need) == need;
+        // a rotation longer than one may leave the window
+        bool ok = ix >= 0 && iy >= 0 && ix < WS - 1 && iy < WS - 1;
+        ok = ok && ((ws->rowmask[iy] >> ix) & need) == need;
         if (fry > 0.0f) ok = ok && (((ws->rowmask[iy + 1] >> ix) & need) == need);
         float tt;
         if (ghost) {
@@ -1014,8 +1018,11 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
                     sh = __fdiv_rn(g.y, a);
                 }
                 const float beta = p.coef32 * a2;
-                // |g| of a few denormals (or infinite): the rotation is not one
-                odd = !(fabsf(ch) <= 1.0001f && fabsf(sh) <= 1.0001f);
+                // |g| of a few denormals (or not finite): the rotation is not one, and may
+                // carry a sample out of the ball's square.  (Correctly rounded, ch^2 + sh^2
+                // is within 3.6e-7 of 1 otherwise.)
+                odd = a > 0.0f && !(__fmaf_rn(ch, ch, __fmul_rn(sh, sh)) <= 1.0000005f);
+                odd = odd || !(a < INFINITY);
                 // group weights e^(-beta g^2), g = |m| = 0..R, shared by the pixel's lanes
                 __syncwarp();
                 if (act)
@@ -1023,7 +1030,7 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
                 __syncwarp();
                 if (act && !odd) {
                     const float *eg = ws->eg[grp];
-                    if (RW == 4 && p.tau >= 2e-6f) rotated_pairs<RW, true>(p, ws, eg, pix, j, G, ch, sh, any, acc);
+                    if (RW == 4 && p.tau >= 6e-6f) rotated_pairs<RW, true>(p, ws, eg, pix, j, G, ch, sh, any, acc);
                     else rotated_pairs<RW, false>(p, ws, eg, pix, j, G, ch, sh, any, acc);
                     if (decide && j == 0)
                         for (int gg = 0; gg <= R; gg++) S_all = __fmaf_rn(eg[gg], p.tab.Dm[gg], S_all);

@@ -70,6 +70,18 @@ def test_guides_of_a_few_denormals(cuda_device):
         _gpu.assert_parity(o, _gpu.gpu_fill(img, labels, g, **kw), labels)
 
 
+def test_rotations_longer_than_one(cuda_device):
+    """Both components of g square to 1.49 units of the smallest denormal, which rounds to
+    one: (g/|g|)^2 sums to 1.49, and the sample (2, -2) lands 3.45 px away."""
+    img, labels = _scene(6)
+    v = np.float32(np.sqrt(1.49 * 2.0 ** -149))
+    rng = np.random.default_rng(3)
+    g = (rng.choice([-1.0, 1.0], (H, W, 2)) * v).astype(np.float32)
+    for kw in (dict(), dict(smart=False), dict(eps=2.9), dict(eps=4.0), dict(eps=5.0)):
+        o = _gpu.oracle_fill(img, labels, g, **kw)
+        _gpu.assert_parity(o, _gpu.gpu_fill(img, labels, g, **kw), labels)
+
+
 def test_colours_that_are_not_finite(cuda_device):
     """A tap of zero weight is not read: an infinite known colour spreads to the pixels
     whose samples use it, with its sign, and to no other."""
