@@ -62,6 +62,7 @@ struct gf_ctx {
     };
     std::vector<Tuned> tuned;
     int max_clusters[3][5] = {};  // co-resident fill clusters by window (4, 5, 8) and size 1, 2, 4, 8, 16 (0: not asked yet)
+    int max_adj[3][5] = {};       // co-resident adjoint clusters by reach (3, 4, 8) and size, likewise
 };
 
 static uint64_t tune_key(int n, const gf_frame *frames, const gf_params *p)
@@ -289,11 +290,16 @@ gf_status gf_create(gf_ctx **out, int device)
     ctx = new gf_ctx();
     ctx->device = device;
     ctx->sm_count = prop.multiProcessorCount;
-    e = cudaFuncSetAttribute((const void *)adj_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) {
-        ctx->last_cuda = (int)e;
-        delete ctx;
-        return GF_ERR_CUDA;
+    for (int rr : {3, 4, 8}) {
+        const void *k = adj_kernel_entry(rr);
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)adj_smem_bytes(rr));
+        if (e != cudaSuccess) {
+            ctx->last_cuda = (int)e;
+            delete ctx;
+            return GF_ERR_CUDA;
+        }
     }
     for (int rw : {4, 5, 8}) {
         const void *k = fill_kernel_ptr(rw);
@@ -1292,43 +1298,55 @@ gf_status gf_fill_backward(gf_ctx *ctx, int n, const gf_adjoint_frame *frames, c
     size_t pos = 0;
     std::vector<int32_t> blk(n + 1);
     int64_t nb = 0;
+    // what starts at zero, in one piece: histograms, step counts, the queue head
     for (int i = 0; i < n; i++) {
-        size_t np = (size_t)frames[i].H * frames[i].W;
+        const size_t np = (size_t)frames[i].H * frames[i].W;
         o_cnt[i] = pos; pos = align_up(pos + 4 * (np + 1), 256);
-        o_start[i] = pos; pos = align_up(pos + 4 * (np + 2), 256);
-        o_order[i] = pos; pos = align_up(pos + 4 * np, 256);
         blk[i] = (int32_t)nb;
         nb += (int64_t)((np + 1023) / 1024);
     }
     blk[n] = (int32_t)nb;
     if (nb >= INT32_MAX / 2) return GF_ERR_ARG;
     const size_t o_K = pos; pos = align_up(pos + 4 * (size_t)n, 256);
+    const size_t o_cur = pos; pos = align_up(pos + 4, 256);
+    const size_t zero_end = pos;
+    for (int i = 0; i < n; i++) {
+        const size_t np = (size_t)frames[i].H * frames[i].W;
+        o_start[i] = pos; pos = align_up(pos + 4 * (np + 2), 256);
+        o_order[i] = pos; pos = align_up(pos + 4 * np, 256);
+    }
     const size_t o_desc = pos; pos = align_up(pos + sizeof(AdjFrameDev) * (size_t)n, 256);
     const size_t o_blk = pos; pos = align_up(pos + 4 * (size_t)(n + 1), 256);
-    const size_t o_cur = pos; pos = align_up(pos + 4, 256);
-    // launch shape: clusters of up to 8 CTAs, one frame per cluster at a time
-    int cs = 8;
-    while (cs > 1 && cs * n > ctx->sm_count) cs >>= 1;
-    int maxc = 0;
-    {
+    // launch shape: a frame per cluster at a time, the largest cluster with which every
+    // frame has its own at once (a frame's reverse sweep is a chain of steps)
+    const int rr = adj_reach((int)std::ceil((double)prm->eps), prm->snap_tau);
+    auto max_clusters = [&](int size) -> int {
+        int *known = nullptr;
+        for (int i = 0; i < 5; i++)
+            if (size == 1 << i) known = &ctx->max_adj[rr == 3 ? 0 : (rr == 4 ? 1 : 2)][i];
+        if (known && *known > 0) return *known;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(cs * 64);
+        cfg.gridDim = dim3(size * 64);
         cfg.blockDim = dim3(CTA_THREADS);
+        cfg.dynamicSmemBytes = adj_smem_bytes(rr);
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = cs;
+        at[0].val.clusterDim.x = size;
         at[0].val.clusterDim.y = 1;
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        while (cs >= 1) {
-            at[0].val.clusterDim.x = cs;
-            cfg.gridDim = dim3(cs * 64);
-            if (cudaOccupancyMaxActiveClusters(&maxc, (const void *)adj_kernel, &cfg) == cudaSuccess && maxc > 0) break;
+        int m = 0;
+        if (cudaOccupancyMaxActiveClusters(&m, adj_kernel_entry(rr), &cfg) != cudaSuccess) {
             cudaGetLastError();
-            cs >>= 1;
+            return 0;
         }
-    }
+        if (known) *known = m;
+        return m;
+    };
+    int cs = 16;
+    while (cs > 1 && max_clusters(cs) < n) cs >>= 1;
+    const int maxc = max_clusters(cs);
     if (maxc <= 0) return GF_ERR_UNSUPPORTED;
     const int nc = std::max(1, std::min(maxc, n));
     const size_t o_cf = pos; pos = align_up(pos + 8 * (size_t)nc, 256);
@@ -1378,14 +1396,8 @@ gf_status gf_fill_backward(gf_ctx *ctx, int n, const gf_adjoint_frame *frames, c
         adj_upload_kernel<<<1, 128, 0, st>>>(ch);
         CK(cudaGetLastError());
     }
-    for (int i = 0; i < n; i++) {
-        size_t np = (size_t)frames[i].H * frames[i].W;
-        CK(cudaMemsetAsync(A + o_cnt[i], 0, 4 * (np + 1), st));
-        CK(cudaMemsetAsync(frames[i].grad_mu, 0, 4, st));
-    }
-    CK(cudaMemsetAsync(A + o_K, 0, 4 * (size_t)n, st));
-    CK(cudaMemsetAsync(A + o_cur, 0, 4, st));
-    const int grid = std::max(1, std::min<int>((int)std::min<int64_t>(nb * 4, INT32_MAX), ctx->sm_count * 8));
+    CK(cudaMemsetAsync(A, 0, zero_end, st));
+    const unsigned grid = (unsigned)nb;
     adj_prep_kernel<<<grid, 256, 0, st>>>(aa);
     CK(cudaGetLastError());
     adj_scan_kernel<<<n, 1024, 0, st>>>(aa);
@@ -1395,6 +1407,7 @@ gf_status gf_fill_backward(gf_ctx *ctx, int n, const gf_adjoint_frame *frames, c
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(nc * cs));
     cfg.blockDim = dim3(CTA_THREADS);
+    cfg.dynamicSmemBytes = adj_smem_bytes(rr);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1403,7 +1416,7 @@ gf_status gf_fill_backward(gf_ctx *ctx, int n, const gf_adjoint_frame *frames, c
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    CK(cudaLaunchKernelEx(&cfg, adj_kernel, aa));
+    CK(launch_adj(rr, cfg, aa));
     return GF_OK;
 }
 

@@ -237,7 +237,10 @@ __global__ void adj_upload_kernel(const __grid_constant__ AdjChunk c);
 __global__ void adj_prep_kernel(const __grid_constant__ AdjArgs a);
 __global__ void adj_scan_kernel(const __grid_constant__ AdjArgs a);
 __global__ void adj_scatter_kernel(const __grid_constant__ AdjArgs a);
-__global__ void adj_kernel(const __grid_constant__ AdjArgs a);
+int adj_reach(int R, float tau);          // rows around a pixel: the kernel's variant
+const void *adj_kernel_entry(int rr);
+size_t adj_smem_bytes(int rr);
+cudaError_t launch_adj(int rr, const cudaLaunchConfig_t &cfg, const AdjArgs &a);
 
 // Descriptor upload by value through kernel parameters: no host staging buffer
 // whose lifetime would have to outlast an asynchronous copy or a graph replay.
