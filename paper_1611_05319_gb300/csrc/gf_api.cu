@@ -184,6 +184,7 @@ void gf::build_tab(float eps, SampleTab &tab)
     for (int s = 0; s < tab.ns; s++) {
         tab.cn[s] = (int8_t)cn[s];
         tab.cm[s] = (int8_t)cm[s];
+        tab.cinv[s] = 1.0 / std::sqrt((double)(cn[s] * cn[s] + cm[s] * cm[s]));
     }
     int pos = 0;
     for (int g = 0; g <= R; g++) {

@@ -304,15 +304,19 @@ __device__ __forceinline__ unsigned long long dilate_nbr(unsigned long long fm, 
     return out;
 }
 
-// FP64 confidence of tile pixel `pix` in the canonical sample order with the
-// oracle's expressions (eqs. weight, confidence); used only inside the FP32
-// guard band.  The whole warp works on one pixel: every lane evaluates the
-// weights of its share of the samples (FP64 runs at a small fraction of the
-// FP32 rate on this part, so the exp/divide work is spread over 32 lanes),
-// then the weights are added in the canonical order exactly as the oracle
-// adds them.  Must be called by all 32 lanes.
+// FP64 confidence of tile pixel `pix` (eqs. weight, confidence) against c; used only
+// inside the FP32 guard band.  The whole warp works on one pixel, every lane on its
+// share of the samples.  First the weights are summed over the lanes in a tree, with
+// the table's reciprocal distances: that decides unless S_rd is within 1e-12 S_all of
+// c S_all, far above the at most 1e-13 by which such sums can differ from any other
+// order's.  Otherwise the weights are added in the canonical order with the oracle's
+// expressions, exactly as the oracle adds them.  FP64 runs at a 64th of the FP32 rate
+// here and a re-check holds up its frame's step: the canonical sums alone, two chains
+// of 28 to 148 additions behind a division and a square root per sample, added 11 us
+// (eps 3) to 25 us (eps 5) to the step; the tree adds 2 to 4 us.  Must be called by all 32
+// lanes.
 template <int RW>
-__device__ bool warp_ready_fp64(const FillParams &p, const WarpSmem<RW> *ws, int pix, bool ghost)
+__device__ __noinline__ bool warp_ready_fp64(const FillParams &p, const WarpSmem<RW> *ws, int pix, bool ghost)
 {
     constexpr int NSLOT = RW == 4 ? 1 : (RW == 5 ? 2 : 5);  // ceil(samples / 32) for ceil(eps) = 3, 4, 7
     const int lane = threadIdx.x & 31;
@@ -328,13 +332,13 @@ __device__ bool warp_ready_fp64(const FillParams &p, const WarpSmem<RW> *ws, int
         }
     }
     const double a2 = __dadd_rn(__dmul_rn((double)gx, (double)gx), __dmul_rn((double)gy, (double)gy));
-    double w[NSLOT];
-    int ok[NSLOT];
+    double e[NSLOT];  // e^-t
+    unsigned ok = 0;  // by slot
+    double A = 0.0, B = 0.0;
 #pragma unroll
     for (int q = 0; q < NSLOT; q++) {
         const int s = q * 32 + lane;
-        w[q] = 0.0;
-        ok[q] = 0;
+        e[q] = 0.0;
         if (s < p.tab.ns) {
             const int n = p.tab.cn[s], m = p.tab.cm[s];
             float ox, oy;
@@ -364,19 +368,40 @@ __device__ bool warp_ready_fp64(const FillParams &p, const WarpSmem<RW> *ws, int
                 const double proj = __dadd_rn(__dmul_rn(-(double)gy, (double)n), __dmul_rn((double)gx, (double)m));
                 t = __dmul_rn(__dmul_rn(p.coef64, proj), proj);
             }
-            w[q] = __ddiv_rn(exp(-t), __dsqrt_rn((double)(n * n + m * m)));
-            ok[q] = rd ? 1 : 0;
+            e[q] = exp(-t);
+            const double w = e[q] * p.tab.cinv[s];
+            A += w;
+            if (rd) {
+                B += w;
+                ok |= 1u << q;
+            }
         }
     }
-    double S_all = 0.0, S_rd = 0.0;
 #pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        A += __shfl_xor_sync(FULL, A, o);
+        B += __shfl_xor_sync(FULL, B, o);
+    }
+    const double d = B - p.c64 * A;
+    if (fabs(d) > 1e-12 * A) return d > 0.0;  // the same on every lane
+    double S_all = 0.0, S_rd = 0.0;
+#pragma unroll 1
     for (int q = 0; q < NSLOT; q++) {
+        const int s = q * 32 + lane;
+        double w = 0.0;
+        if (s < p.tab.ns) {
+            const int n = p.tab.cn[s], m = p.tab.cm[s];
+            double eq = e[0];
+#pragma unroll
+            for (int i = 1; i < NSLOT; i++) eq = q == i ? e[i] : eq;
+            w = __ddiv_rn(eq, __dsqrt_rn((double)(n * n + m * m)));
+        }
         for (int src = 0; src < 32; src++) {
-            const double wv = __shfl_sync(FULL, w[q], src);
-            const int okv = __shfl_sync(FULL, ok[q], src);
+            const double wv = __shfl_sync(FULL, w, src);
+            const unsigned okv = __shfl_sync(FULL, ok, src);
             if (q * 32 + src < p.tab.ns) {
                 S_all = __dadd_rn(S_all, wv);
-                if (okv) S_rd = __dadd_rn(S_rd, wv);
+                if ((okv >> q) & 1u) S_rd = __dadd_rn(S_rd, wv);
             }
         }
     }
@@ -849,19 +874,25 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
         }
     }
     const int wx0 = x0 - RW, wy0 = y0 - RW;
-    // State window.  With WS = 16 a lane holds 4 columns of 2 rows (lane = 4 row +
-    // column group): one 16-byte load each when the row width is a multiple of 4 and
-    // the state array is aligned (4 columns are then wholly inside or wholly outside
-    // the frame), else 4 plain loads.  Other widths: one column per lane and row.
-    constexpr bool Q4 = WS == 16;
-    int32_t sv[Q4 ? 1 : WS];
-    int4 sq[2];
-    if (Q4) {
+    // State window: 16-byte loads of 4 columns when the row width is a multiple of 4 and
+    // the state array is aligned (4 columns are then wholly inside or wholly outside the
+    // frame), else 4 plain loads.  RW = 4: 4 quads of 2 x 8 rows from column x0 - 4; wider
+    // windows: 6 quads of 4 rows at a time from column x0 - 8, of which the window is a part
+    // (one column per lane and row took 4,400 to 6,800 cycles a tile to issue, with the
+    // colour window by divisions, and takes 2,200 to 2,900).
+    constexpr int QW = RW == 4 ? 4 : 8;           // lanes per row
+    constexpr int QR = 32 / QW;                   // rows per load
+    constexpr int QN = (WS + QR - 1) / QR;        // loads
+    constexpr int QX = RW == 4 ? 4 : 8;           // columns left of the tile
+    int4 sq[QN];
+    {
         const bool vec = (W & 3) == 0 && ((uintptr_t)F.shell & 15u) == 0;
+        const int gx = x0 - QX + 4 * (lane & (QW - 1));
+        const bool qin = RW == 4 || (lane & 7) < 6;
 #pragma unroll
-        for (int i = 0; i < 2; i++) {
-            const int gx = wx0 + 4 * (lane & 3), gy = wy0 + (lane >> 2) + 8 * i;
-            const bool rin = gy >= 0 && gy < H;
+        for (int i = 0; i < QN; i++) {
+            const int r = lane / QW + QR * i, gy = wy0 + r;
+            const bool rin = qin && r < WS && gy >= 0 && gy < H;
             if (vec) {
                 sq[i] = (rin && gx >= 0 && gx < W) ? ld(reinterpret_cast<const int4 *>(&F.shell[(size_t)gy * W + gx]))
                                                    : make_int4(SH_OUTSIDE, SH_OUTSIDE, SH_OUTSIDE, SH_OUTSIDE);
@@ -872,13 +903,6 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
                     e[b] = (rin && gx + b >= 0 && gx + b < W) ? ld(&F.shell[(size_t)gy * W + gx + b]) : SH_OUTSIDE;
                 sq[i] = make_int4(e[0], e[1], e[2], e[3]);
             }
-        }
-    } else {
-#pragma unroll
-        for (int r = 0; r < (Q4 ? 1 : WS); r++) {
-            int gx = wx0 + lane, gy = wy0 + r;
-            sv[r] = (lane < WS && gx >= 0 && gy >= 0 && gx < W && gy < H) ? ld(&F.shell[(size_t)gy * W + gx])
-                                                                           : SH_OUTSIDE;
         }
     }
     float2 gv[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -901,10 +925,19 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
                 cp_async16(&ws->col[(r0 + 2 * i) * 16 + c], &F.rgba[(size_t)gy * W + wx0 + c]);
         }
     } else {
-        for (int e = lane; e < WS * WS; e += 32) {
-            int r = e / WS, c = e - r * WS;
-            int gx = wx0 + c, gy = wy0 + r;
-            if (gx >= 0 && gy >= 0 && gx < W && gy < H) cp_async16(&ws->col[e], &F.rgba[(size_t)gy * W + gx]);
+        // blocks of CR rows x CW columns (WS is a multiple of CW), one element per lane
+        constexpr int CW = WS % 8 == 0 ? 8 : 6, CR = 32 / CW;
+        const int r0 = lane / CW, c0 = lane - r0 * CW;
+        const float4 *src = F.rgba + ((ptrdiff_t)(wy0 + r0) * W + wx0 + c0);
+        float4 *dst = &ws->col[r0 * WS + c0];
+#pragma unroll
+        for (int i = 0; i < (WS + CR - 1) / CR; i++) {
+            const bool rin = r0 < CR && r0 + CR * i < WS && (unsigned)(wy0 + r0 + CR * i) < (unsigned)H;
+#pragma unroll
+            for (int c = 0; c < WS / CW; c++)
+                if (rin && (unsigned)(wx0 + c0 + CW * c) < (unsigned)W)
+                    cp_async16(dst + CR * WS * i + CW * c, src + CW * c);
+            src += (ptrdiff_t)CR * W;
         }
     }
 
@@ -924,23 +957,16 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
     if (cand == 0) return;
 
     // ---- readable bits of the window by ballot; guide vectors of the candidates
-    if (Q4) {
-        // each lane's 4 readable bits at column 4 (lane & 3), OR-ed over the 4 lanes of a row
+    // each lane's 4 readable bits at its quad's columns, OR-ed over the lanes of a row
 #pragma unroll
-        for (int i = 0; i < 2; i++) {
-            uint32_t v = (readable_at(sq[i].x, k) ? 1u : 0u) | (readable_at(sq[i].y, k) ? 2u : 0u) |
-                         (readable_at(sq[i].z, k) ? 4u : 0u) | (readable_at(sq[i].w, k) ? 8u : 0u);
-            v <<= 4 * (lane & 3);
-            v |= __shfl_xor_sync(FULL, v, 1);
-            v |= __shfl_xor_sync(FULL, v, 2);
-            if ((lane & 3) == 0) ws->rowmask[(lane >> 2) + 8 * i] = v;
-        }
-    } else {
+    for (int i = 0; i < QN; i++) {
+        const int r = lane / QW + QR * i;
+        uint32_t v = (readable_at(sq[i].x, k) ? 1u : 0u) | (readable_at(sq[i].y, k) ? 2u : 0u) |
+                     (readable_at(sq[i].z, k) ? 4u : 0u) | (readable_at(sq[i].w, k) ? 8u : 0u);
+        v = RW == 4 || (lane & 7) < 6 ? v << (4 * (lane & (QW - 1))) : 0u;
 #pragma unroll
-        for (int r = 0; r < (Q4 ? 1 : WS); r++) {
-            unsigned b = __ballot_sync(FULL, readable_at(sv[r], k));
-            if (lane == 0) ws->rowmask[r] = b;
-        }
+        for (int o = 1; o < QW; o <<= 1) v |= __shfl_xor_sync(FULL, v, o);
+        if ((lane & (QW - 1)) == 0 && r < WS) ws->rowmask[r] = (v >> (QX - RW)) & ((1u << WS) - 1u);
     }
     if (MODE != STALL) {
 #pragma unroll
@@ -993,7 +1019,7 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
     if (np) {
         cp_async_wait_all();
         __syncwarp();
-        const int2 lanes = c_lanes[min(np, 17)];
+        const int2 lanes = c_lanes[p.tab.ns <= 32 ? max(min(np, 17), 2) : min(np, 17)];
         const int G = lanes.x, per = 32 / G;
         const int grp = (lane * lanes.y) >> 8, j = lane - grp * G;  // lane / G, lane % G
         const bool decide = MODE != STALL && smart;
@@ -1046,14 +1072,12 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
                 const float c0 = __shfl_down_sync(FULL, axy.x, o), c1 = __shfl_down_sync(FULL, axy.y, o);
                 const float c2 = __shfl_down_sync(FULL, azw.x, o), c3 = __shfl_down_sync(FULL, azw.y, o);
                 const bool in = j + o < G;
-                if (in) {
-                    weight_add(S_rd, S_lo, s0);
-                    S_lo += s1;
-                    axy.x += c0;
-                    axy.y += c1;
-                    azw.x += c2;
-                    azw.y += c3;
-                }
+                weight_add(S_rd, S_lo, in ? s0 : 0.f);
+                S_lo += in ? s1 : 0.f;
+                axy.x += in ? c0 : 0.f;
+                axy.y += in ? c1 : 0.f;
+                azw.x += in ? c2 : 0.f;
+                azw.y += in ? c3 : 0.f;
                 if (!plain) {
                     const float a1 = __shfl_down_sync(FULL, S_all, o);
                     const bool an = __shfl_down_sync(FULL, (int)any, o) != 0;

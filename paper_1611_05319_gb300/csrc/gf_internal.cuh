@@ -51,6 +51,7 @@ struct SampleTab {
     float invd[MAX_SAMPLES];     // 1 / sqrt(n^2 + m^2)
     int8_t cn[MAX_SAMPLES];      // canonical order
     int8_t cm[MAX_SAMPLES];
+    double cinv[MAX_SAMPLES];    // 1 / sqrt(n^2 + m^2)
 };
 
 // Per-warp shared memory of the fill kernel: the staged (8 + 2 RW)^2 window

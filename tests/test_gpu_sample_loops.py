@@ -36,6 +36,17 @@ def test_every_ball(cuda_device, eps, kw):
         _gpu.assert_parity(o, _gpu.gpu_fill(img, labels, g, eps=eps, **kg), labels)
 
 
+@pytest.mark.parametrize("width", [80, 84, 85, 96])
+@pytest.mark.parametrize("eps", [3.0, 4.0, 5.0, 7.0])
+def test_windows_at_every_width(cuda_device, width, eps):
+    """16-byte and plain loads of the state window, tiles cut by the right border."""
+    hole = _gpu.hole_blobs(H, width, 12, n=14, rmin=1, rmax=7, margin=4)
+    img, g = polygon_image(H, width, 7, 2), random_guide(H, width, 6)
+    for kw in (dict(), dict(ghost=False)):
+        o = _gpu.oracle_fill(img, labels_from(hole), g, eps=eps, **kw)
+        _gpu.assert_parity(o, _gpu.gpu_fill(img, labels_from(hole), g, eps=eps, **kw), labels_from(hole))
+
+
 @pytest.mark.parametrize("n", list(range(1, 18)) + [23, 32, 33, 48, 64])
 def test_front_pixels_per_tile(cuda_device, n):
     """n isolated hole pixels or short rows of them in one 8x8 tile."""
