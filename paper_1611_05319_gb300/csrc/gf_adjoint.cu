@@ -205,6 +205,10 @@ __device__ __forceinline__ SampleGeo sample_geo(const AdjArgs &a, const AdjFrame
     return g;
 }
 
+__device__ __forceinline__ float4 operator-(float4 a, float4 b)
+{
+    return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+}
 __device__ __forceinline__ float dot4(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 
 __device__ __forceinline__ void red_add4(float4 *p, float4 v)
@@ -216,7 +220,7 @@ __device__ __forceinline__ void red_add4(float4 *p, float4 v)
 // the pixels whose rotation is not one (|g| of a few denormals, or not finite).  Must
 // be called by all 32 lanes.
 __device__ __noinline__ void adj_pixel_general(const AdjArgs &a, const AdjFrameDev &F, int p, int k, bool stall, bool act, int G,
-                          int j, float &mu_acc)
+                          int j, double &mu_acc)
 {
     const int x = p % F.W, y = p / F.W;
     float4 ub = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -327,7 +331,7 @@ __device__ __noinline__ void adj_pixel_general(const AdjArgs &a, const AdjFrameD
     if (act && j == 0) {
         F.grad_phi[p] = has_dir ? S4 : 0.f;
         F.grad_in[p] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!stall) mu_acc += S1 - S2 * S3;
+        if (!stall) mu_acc += (double)(S1 - S2 * S3);
     }
 }
 
@@ -346,6 +350,7 @@ struct AdjPix {
     float ch, sh;   // rotation
     float a2;       // |g|^2
     float inv;      // 1 / sum of the readable weights, 0 when there is none
+    float4 u;       // the pixel's own output (0 when it is not finite)
     int least;      // smallest readable |m|
     bool rot;       // not a stall step
     bool odd;       // to be done by adj_pixel_general
@@ -397,6 +402,7 @@ __device__ __forceinline__ AdjPix adj_prepare(const AdjArgs &a, const AdjFrameDe
     px.sh = 0.f;
     px.inv = 0.f;
     px.least = 0;
+    px.u = make_float4(0.f, 0.f, 0.f, 0.f);
     px.odd = false;
     const int W = F.W, H = F.H, R = a.tab.R;
     __syncwarp();  // the previous batch's rows and weights have been read
@@ -405,6 +411,9 @@ __device__ __forceinline__ AdjPix adj_prepare(const AdjArgs &a, const AdjFrameDe
         const int x = px.p % W, y = px.p / W;
         float2 g = make_float2(0.f, 0.f);
         if (!stall) g = __ldg(&F.guide[px.p]);
+        px.u = __ldg(&F.out[px.p]);
+        if (!(fabsf(px.u.x) + fabsf(px.u.y) + fabsf(px.u.z) + fabsf(px.u.w) < INFINITY))
+            px.u = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int r = j; r < N; r += G) {
             const int yy = y + r - RR;
             const bool rin = yy >= 0 && yy < H;
@@ -471,7 +480,7 @@ __device__ __forceinline__ AdjPix adj_prepare(const AdjArgs &a, const AdjFrameDe
 // Scatter, angle and mu terms of a prepared batch.  Called by all 32 lanes.
 template <int RR>
 __device__ __forceinline__ void adj_apply(const AdjArgs &a, const AdjFrameDev &F, const AdjWarp<RR> *aw, const float4 *pairs,
-                                          const AdjPix &px, int k, int G, int grp, int j, float &mu_acc)
+                                          const AdjPix &px, int k, int G, int grp, int j, double &mu_acc)
 {
     if (__any_sync(AFULL, px.odd)) {  // whole batch: rare
         adj_pixel_general(a, F, px.p < 0 ? 0 : px.p, k, !px.rot, px.p >= 0, G, j, mu_acc);
@@ -512,8 +521,10 @@ __device__ __forceinline__ void adj_apply(const AdjArgs &a, const AdjFrameDev &F
 #pragma unroll
             for (int h = 0; h < 2; h++) {
                 if (!(h ? c.ok2 : c.ok1)) continue;
-                const float d00 = dot4(v[h][0], ub), d10 = dot4(v[h][1], ub), d01 = dot4(v[h][2], ub),
-                            d11 = dot4(v[h][3], ub);
+                // relative to the pixel's own value, the average of the samples: constants
+                // cancel in the angle and mu terms, and taken off first they cost no digits
+                const float d00 = dot4(v[h][0] - px.u, ub), d10 = dot4(v[h][1] - px.u, ub),
+                            d01 = dot4(v[h][2] - px.u, ub), d11 = dot4(v[h][3] - px.u, ub);
                 float vu = gx * gy * d00;
                 if (c.hx) vu += c.frx * gy * d10;
                 if (c.hy) vu += gx * c.fry * d01;
@@ -554,7 +565,7 @@ __device__ __forceinline__ void adj_apply(const AdjArgs &a, const AdjFrameDev &F
     if (act && j == 0) {
         F.grad_phi[px.p] = has_dir ? S4 : 0.f;
         F.grad_in[px.p] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (px.rot) mu_acc += S1 - S2 * S3;
+        if (px.rot) mu_acc += (double)(S1 - S2 * S3);
     }
 }
 
@@ -590,7 +601,7 @@ __global__ void __launch_bounds__(CTA_THREADS, 1) adj_kernel(const __grid_consta
         __syncthreads();
         const AdjFrameDev &F = s_frame;
         const int K = __ldcg(F.K);
-        float mu_acc = 0.f;
+        double mu_acc = 0.0;  // signed terms of all of the frame's pixels
         // step k's first batch, prepared while the barrier of step k + 1 is pending
         int b0 = 0, b1 = 0, G = 2, per = 16, grp = 0, j = 0;
         bool stall = false;
@@ -619,10 +630,12 @@ __global__ void __launch_bounds__(CTA_THREADS, 1) adj_kernel(const __grid_consta
                 prepare(k - 1);
             }
         }
-        float wsum = mu_acc;
+        double wsum = mu_acc;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(AFULL, wsum, o);
-        if (lane == 0 && wsum != 0.f) atomicAdd(&F.grad_mu[0], wsum);
+        if (lane == 0 && wsum != 0.0) atomicAdd(F.mu_sum, wsum);
+        cluster.sync();
+        if (crank == 0 && threadIdx.x == 0) atomicAdd(F.grad_mu, (float)__ldcg(F.mu_sum));
         __syncthreads();
     }
 }

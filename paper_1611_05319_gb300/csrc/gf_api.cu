@@ -1299,7 +1299,7 @@ gf_status gf_fill_backward(gf_ctx *ctx, int n, const gf_adjoint_frame *frames, c
     size_t pos = 0;
     std::vector<int32_t> blk(n + 1);
     int64_t nb = 0;
-    // what starts at zero, in one piece: histograms, step counts, the queue head
+    // what starts at zero, in one piece: histograms, step counts, the queue head, mu sums
     for (int i = 0; i < n; i++) {
         const size_t np = (size_t)frames[i].H * frames[i].W;
         o_cnt[i] = pos; pos = align_up(pos + 4 * (np + 1), 256);
@@ -1310,6 +1310,7 @@ gf_status gf_fill_backward(gf_ctx *ctx, int n, const gf_adjoint_frame *frames, c
     if (nb >= INT32_MAX / 2) return GF_ERR_ARG;
     const size_t o_K = pos; pos = align_up(pos + 4 * (size_t)n, 256);
     const size_t o_cur = pos; pos = align_up(pos + 4, 256);
+    const size_t o_mu = pos; pos = align_up(pos + 8 * (size_t)n, 256);
     const size_t zero_end = pos;
     for (int i = 0; i < n; i++) {
         const size_t np = (size_t)frames[i].H * frames[i].W;
@@ -1386,6 +1387,7 @@ gf_status gf_fill_backward(gf_ctx *ctx, int n, const gf_adjoint_frame *frames, c
             d.grad_in = (float4 *)f.grad_in;
             d.grad_phi = f.grad_phi;
             d.grad_mu = f.grad_mu;
+            d.mu_sum = (double *)(A + o_mu) + (c0 + i);
             d.cnt = (int32_t *)(A + o_cnt[c0 + i]);
             d.start = (int32_t *)(A + o_start[c0 + i]);
             d.order = (int32_t *)(A + o_order[c0 + i]);

@@ -210,6 +210,7 @@ struct AdjFrameDev {
     float4 *grad_in;
     float *grad_phi;
     float *grad_mu;           // one float per frame
+    double *mu_sum;           // its sum (zeroed)
     int32_t *cnt;             // [H*W+1]: histogram, then scatter cursor
     int32_t *start;           // [H*W+2]
     int32_t *order;           // [H*W]
