@@ -924,21 +924,28 @@ static gf_status guidance_impl(gf_ctx *ctx, DevBuf &garena, int n, const gf_spli
     cudaError_t e = cudaSetDevice(ctx->device);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     cudaStream_t st = (cudaStream_t)stream;
-    std::vector<size_t> off_cnt(n), off_list(n), off_seg(n);
+    std::vector<size_t> off_cnt(n), off_list(n), off_seg(n), off_segp(n);
     size_t pos = 0;
     int64_t tot_pts = 0, tot_bins = 0;
+    for (int i = 0; i < n; i++) {  // the bin counts, in one piece: they start at zero
+        const size_t nb = (size_t)((frames[i].W + BIN - 1) / BIN) * ((frames[i].H + BIN - 1) / BIN);
+        off_cnt[i] = pos; pos = align_up(pos + 4 * nb, 256);
+    }
+    const size_t cnt_end = pos;
     for (int i = 0; i < n; i++) {
         int NBX = (frames[i].W + BIN - 1) / BIN, NBY = (frames[i].H + BIN - 1) / BIN;
-        off_cnt[i] = pos; pos = align_up(pos + 4 * (size_t)NBX * NBY, 256);
+        const size_t np = (size_t)std::max(frames[i].n_points, 1);
         off_list[i] = pos; pos = align_up(pos + 4 * (size_t)NBX * NBY * BIN_CAP, 256);
-        off_seg[i] = pos; pos = align_up(pos + 64 * (size_t)std::max(frames[i].n_points, 1), 256);
+        off_seg[i] = pos; pos = align_up(pos + 64 * np, 256);
+        off_segp[i] = pos; pos = align_up(pos + sizeof(SegPair) * np, 256);
         tot_pts += frames[i].n_points;
         tot_bins += (int64_t)NBX * NBY;
     }
-    if (tot_pts >= INT32_MAX || tot_bins >= INT32_MAX) return GF_ERR_ARG;
+    if (tot_pts >= INT32_MAX || tot_bins >= INT32_MAX - 8) return GF_ERR_ARG;
     const size_t off_desc = pos; pos = align_up(pos + sizeof(SplineFrameDev) * (size_t)n, 256);
     const size_t off_po = pos; pos = align_up(pos + 4 * (size_t)(n + 1), 256);
     const size_t off_bo = pos; pos = align_up(pos + 4 * (size_t)(n + 1), 256);
+    const size_t off_exps = pos; pos = align_up(pos + sizeof(GuideExp), 256);
     gf_status s = ensure(ctx, garena, pos);
     if (s != GF_OK) return s;
     char *A = (char *)garena.ptr;
@@ -959,22 +966,21 @@ static gf_status guidance_impl(gf_ctx *ctx, DevBuf &garena, int n, const gf_spli
         d.bin_count = (int32_t *)(A + off_cnt[i]);
         d.bin_list = (int32_t *)(A + off_list[i]);
         d.seg64 = (double *)(A + off_seg[i]);
+        d.segp = (SegPair *)(A + off_segp[i]);
+        d.weight = f.weight;
         hd[i] = d;
         hpo[i] = (int32_t)pp; hbo[i] = (int32_t)bb;
         pp += f.n_points;
         bb += (int64_t)d.NBX * d.NBY;
     }
     hpo[n] = (int32_t)pp; hbo[n] = (int32_t)bb;
-    // counts must be zero; lists need no clearing
-    for (int i = 0; i < n; i++) {
-        size_t nbins = (size_t)hd[i].NBX * hd[i].NBY;
-        CK(cudaMemsetAsync(A + off_cnt[i], 0, 4 * nbins, st));
-    }
+    CK(cudaMemsetAsync(A, 0, cnt_end, st));  // lists need no clearing
     for (int c0 = 0; c0 < n; c0 += DESC_CHUNK) {
         static thread_local SplineChunk ch;
         ch.dst_frames = (SplineFrameDev *)(A + off_desc);
         ch.dst_po = (int32_t *)(A + off_po);
         ch.dst_bo = (int32_t *)(A + off_bo);
+        ch.dst_exps = (GuideExp *)(A + off_exps);
         ch.first = c0;
         ch.count = std::min(DESC_CHUNK, n - c0);
         ch.last_chunk = (c0 + ch.count == n) ? 1 : 0;
@@ -996,24 +1002,15 @@ static gf_status guidance_impl(gf_ctx *ctx, DevBuf &garena, int n, const gf_spli
     ga.total_bins = (int32_t)bb;
     ga.eta = eta;
     ga.k2 = 1.0 / (2.0 * (double)eta * (double)eta);
+    ga.k2p = pair_of(ga.k2);
+    ga.ieta = 1.0f / eta;
+    ga.exps = (const GuideExp *)(A + off_exps);
     if (pp > 0) {
         bin_kernel<<<(unsigned)((pp + 255) / 256), 256, 0, st>>>(ga, (int)pp);
         CK(cudaGetLastError());
-        for (int c0 = 0; c0 < n; c0 += DESC_CHUNK) {
-            WeightChunk wc;
-            wc.first = c0;
-            wc.count = std::min(DESC_CHUNK, n - c0);
-            bool any = false;
-            for (int i = 0; i < wc.count; i++) {
-                wc.w[i] = frames[c0 + i].n_points > 1 ? frames[c0 + i].weight : nullptr;
-                any = any || wc.w[i];
-            }
-            if (!any) continue;
-            spline_weight_kernel<<<(unsigned)wc.count, 256, 0, st>>>(ga, wc);
-            CK(cudaGetLastError());
-        }
     }
-    guide_kernel<<<(unsigned)bb, 256, 0, st>>>(ga);
+    // a warp per 8-row strip of four 32x32 bins, eight warps a CTA: eight bins
+    guide_kernel<<<(unsigned)((bb + 7) / 8), 256, 0, st>>>(ga);
     CK(cudaGetLastError());
     return GF_OK;
 }

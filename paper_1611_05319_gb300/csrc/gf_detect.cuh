@@ -113,11 +113,4 @@ __global__ void detect_accept_kernel(const __grid_constant__ DetectArgs a);
 __global__ void detect_scan_kernel(const __grid_constant__ DetectArgs a);
 __global__ void detect_write_kernel(const __grid_constant__ DetectArgs a);
 
-// per-spline weights of a guide-field request: frames [first, first + count)
-struct WeightChunk {
-    const float *w[DESC_CHUNK];
-    int32_t first, count;
-};
-__global__ void spline_weight_kernel(const __grid_constant__ GuideArgs a, const __grid_constant__ WeightChunk c);
-
 }  // namespace gf

@@ -10,16 +10,24 @@
 //                 appended to every 32x32-pixel bin its bounding box, grown by
 //                 3 eta + 1 px, overlaps (so no segment within 3 eta of a pixel
 //                 is missed, FP32 rounding included);
-//   guide_kernel  one CTA per bin: bins without hole pixels end after one
-//                 load per row; otherwise the bin's segments are staged in
-//                 shared memory and each hole pixel takes the nearest one.  A
-//                 bin whose list overflowed scans all segments of its frame.
+//   guide_kernel  one CTA per eight bins, a warp at a time per strip of 8 rows
+//                 of a bin that holds hole pixels: the bin's segments are
+//                 staged in shared memory 32 at a time and each hole pixel
+//                 takes the nearest one.  A bin whose list overflowed scans
+//                 all segments of its frame.
 // The nearest-segment choice and the 3-eta cut use a fixed FP32 expression
 // with no contraction (ties: lowest segment index), so the decision does not
-// depend on the machine; the returned value is evaluated in FP64 for the
-// chosen segment and rounded once to FP32.
+// depend on the machine; the returned value is the FP64 evaluation's for the
+// chosen segment, rounded once to FP32 (formed in pairs of FP32 numbers where
+// those settle the rounding, gf_guide_math.cuh).
+//
+// guide_kernel was bound by FP64 on the SMs with the most hole pixels, with one CTA
+// per bin: 329 us on 32 frames of 1920 x 1080 (2.7 M hole pixels).  In pairs, with the
+// same CTAs' work dealt to warps, 241 us; with the value evaluated in one place instead
+// of unrolled per pixel, which kept the instruction cache missing, and the strips taken
+// by whichever warp is free, 129 us.
 
-#include "gf_detect.cuh"
+#include "gf_internal.cuh"
 
 namespace gf {
 
@@ -30,6 +38,12 @@ __global__ void upload_splines_kernel(const __grid_constant__ SplineChunk c)
         c.dst_po[c.first + i] = c.po[i];
         c.dst_bo[c.first + i] = c.bo[i];
     }
+    if (c.first == 0)
+        for (int j = threadIdx.x; j < GUIDE_EXP; j += blockDim.x) {
+            const Pair e = pair_of(exp(-(double)j / 32.0));
+            c.dst_exps->h[j] = e.h;
+            c.dst_exps->l[j] = e.l;
+        }
     if (threadIdx.x == 0 && c.last_chunk) {
         c.dst_po[c.first + c.count] = c.po[c.count];
         c.dst_bo[c.first + c.count] = c.bo[c.count];
@@ -72,14 +86,23 @@ __global__ void __launch_bounds__(256) bin_kernel(const __grid_constant__ GuideA
         const double dvx = __dsub_rn((double)B.x, ax), dvy = __dsub_rn((double)B.y, ay);
         const double len = __dsqrt_rn(__dadd_rn(__dmul_rn(dvx, dvx), __dmul_rn(dvy, dvy)));
         double *s = F.seg64 + 8 * (size_t)i;
+        const double il = __ddiv_rn(1.0, __dmul_rn(len, len));
+        const double tx = __ddiv_rn(dvx, len), ty = __ddiv_rn(dvy, len);
+        const float sw = F.weight ? __ldg(&F.weight[lo]) : 1.0f;
         s[0] = ax;
         s[1] = ay;
         s[2] = dvx;
         s[3] = dvy;
-        s[4] = __ddiv_rn(1.0, __dmul_rn(len, len));
-        s[5] = __ddiv_rn(dvx, len);
-        s[6] = __ddiv_rn(dvy, len);
-        s[7] = 1.0;  // the spline's weight, set by spline_weight_kernel when given
+        s[4] = il;
+        s[5] = tx;
+        s[6] = ty;
+        s[7] = (double)sw;
+        const Pair px = pair_of(dvx), py = pair_of(dvy), pi = pair_of(il), tpx = pair_of(tx), tpy = pair_of(ty);
+        float4 *d = reinterpret_cast<float4 *>(F.segp + i);
+        d[0] = make_float4(A.x, A.y, px.h, py.h);  // px.h and py.h are vx and vy
+        d[1] = make_float4(__fdiv_rn(1.0f, l2), px.l, py.l, pi.h);
+        d[2] = make_float4(pi.l, tpx.h, tpx.l, tpy.h);
+        d[3] = make_float4(tpy.l, sw, 0.f, 0.f);
     }
     float grow = 3.0f * a.eta + 1.0f;
     float xmin = fminf(A.x, B.x) - grow, xmax = fmaxf(A.x, B.x) + grow;
@@ -116,187 +139,220 @@ __device__ __forceinline__ uint32_t hole4(uint32_t w)
     return ((r >> 7) & 1u) | ((r >> 14) & 2u) | ((r >> 21) & 4u) | ((r >> 28) & 8u);
 }
 
-struct BinSegs {
-    float4 av[BIN_CAP];   // a.x, a.y, v.x, v.y
-    float inv_l2[BIN_CAP];
-    int id[BIN_CAP];      // global segment index (ties go to the lowest)
+constexpr int GUIDE_WARPS = 8;
+constexpr int STRIP = 8;  // rows of a bin per warp
+
+struct GuideWarp {
+    float4 av[32];          // segments staged: a.x, a.y, v.x, v.y
+    float2 ilid[32];        // 1/|v|^2, segment index (as bits)
+    short holes[BIN * STRIP];
+    int seg[BIN * STRIP];   // the nearest segment of each hole pixel, -1: none within 3 eta
 };
 
-// Nearest segment of P hole pixels per thread (pixels q = tid + 256 j): the
-// bin's segments form the outer loop, so each is read from shared memory once
-// per thread.
-template <int P>
-__device__ __forceinline__ void nearest_in_bin(const BinSegs &sg, int nloc, const short *holes, int nh, int x0, int y0,
-                                               float *best, int *bi)
+// The FP64 evaluation: t = ((x - a).v) / |v|^2 clamped, d^2 = |x - a - t v|^2, g = (v/|v|)
+// e^(-d^2/(2 eta^2)), with the reciprocals 1/|v|^2 and 1/(2 eta^2) precomputed in FP64.
+__device__ __noinline__ float2 guide_value64(const double *s, int x, int y, double k2)
 {
-    float px[P], py[P];
+    const double ax = __ldcg(&s[0]), ay = __ldcg(&s[1]), vx = __ldcg(&s[2]), vy = __ldcg(&s[3]);
+    const double inv_l2 = __ldcg(&s[4]), tx = __ldcg(&s[5]), ty = __ldcg(&s[6]), sw = __ldcg(&s[7]);
+    const double wx = __dsub_rn((double)x, ax), wy = __dsub_rn((double)y, ay);
+    double t = __dmul_rn(__dadd_rn(__dmul_rn(wx, vx), __dmul_rn(wy, vy)), inv_l2);
+    if (t < 0.0) t = 0.0;
+    if (t > 1.0) t = 1.0;
+    const double qx = __dsub_rn(wx, __dmul_rn(t, vx)), qy = __dsub_rn(wy, __dmul_rn(t, vy));
+    const double d2 = __dadd_rn(__dmul_rn(qx, qx), __dmul_rn(qy, qy));
+    const double ev = exp(-__dmul_rn(d2, k2));
+    return make_float2((float)__dmul_rn(__dmul_rn(tx, ev), sw), (float)__dmul_rn(__dmul_rn(ty, ev), sw));
+}
+
+// The nearest segments of the strip's hole pixels, P per lane (pixels q = lane + 32 j),
+// the segments in the outer loop so that each is read from shared memory once per lane.
+template <int P>
+__device__ __forceinline__ void nearest_segments(const GuideArgs &a, const SplineFrameDev &F, GuideWarp *gw, int b, int cnt,
+                                             int x0, int y0, int nh, float4 box)
+{
+    const int lane = threadIdx.x & 31;
+    float px[P], py[P], best[P];
+    int bi[P];
 #pragma unroll
     for (int j = 0; j < P; j++) {
-        const int q = threadIdx.x + 256 * j;
-        const int e = q < nh ? holes[q] : 0;
+        const int q = lane + 32 * j;
+        const int e = q < nh ? gw->holes[q] : 0;
         px[j] = (float)(x0 + (e & (BIN - 1)));
         py[j] = (float)(y0 + (e >> 5));
         best[j] = INFINITY;
         bi[j] = 0x7fffffff;
     }
-    for (int s = 0; s < nloc; s++) {
-        const float4 S = sg.av[s];
-        const float il = sg.inv_l2[s];
-        const int id = sg.id[s];
-#pragma unroll
-        for (int j = 0; j < P; j++) {
-            const float d2 = seg_d2(px[j], py[j], S.x, S.y, S.z, S.w, il);
-            if (d2 < best[j] || (d2 == best[j] && id < bi[j])) {
-                best[j] = d2;
-                bi[j] = id;
+    if (cnt <= BIN_CAP) {
+        for (int s0 = 0; s0 < cnt; s0 += 32) {
+            __syncwarp();  // the previous segments have been read
+            // only segments that come within 3 eta of the hole pixels' box matter (one more
+            // px for FP32's rounding, as for the bins): about half of the bin's
+            bool keep = false;
+            int i = 0;
+            float4 S0 = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (s0 + lane < cnt) {
+                i = __ldg(&F.bin_list[(size_t)b * BIN_CAP + s0 + lane]);
+                S0 = __ldg(reinterpret_cast<const float4 *>(F.segp + i));
+                const float ex = S0.x + S0.z, ey = S0.y + S0.w;
+                keep = !(fmaxf(S0.x, ex) < box.x || fminf(S0.x, ex) > box.y || fmaxf(S0.y, ey) < box.z ||
+                         fminf(S0.y, ey) > box.w);
             }
-        }
-    }
-}
-
-// One CTA per 32x32-pixel bin.  Lanes 0-3 of each warp read one row of the bin's
-// labels each (two 16-byte loads where the row is aligned and inside the frame)
-// into a 32-bit hole mask; a bin without hole pixels ends there.  Otherwise the
-// bin's segments are staged in shared memory with their reciprocal lengths, the
-// hole pixels are compacted, and each thread takes the nearest segment of up to
-// four of them.
-__global__ void __launch_bounds__(256) guide_kernel(const __grid_constant__ GuideArgs a)
-{
-    __shared__ BinSegs sg;
-    __shared__ short holes_s[BIN * BIN];
-    __shared__ int wtot[8];
-    const int gb = blockIdx.x;
-    const int f = find_frame(a.bin_offset, a.n_frames, gb);
-    const SplineFrameDev &F = a.frames[f];
-    const int b = gb - __ldg(&a.bin_offset[f]);
-    const int bx = b % F.NBX, by = b / F.NBX;
-    const int x0 = bx * BIN, y0 = by * BIN;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = warp * 4 + lane;  // the bin row of lanes 0-3
-    uint32_t hm = 0u;
-    if (lane < 4 && y0 + r < F.H) {
-        const uint8_t *row = F.labels + (size_t)(y0 + r) * F.W + x0;
-        if (x0 + BIN <= F.W && (reinterpret_cast<uintptr_t>(row) & 15u) == 0) {
-            const uint4 q0 = __ldg(reinterpret_cast<const uint4 *>(row));
-            const uint4 q1 = __ldg(reinterpret_cast<const uint4 *>(row) + 1);
-            hm = hole4(q0.x) | (hole4(q0.y) << 4) | (hole4(q0.z) << 8) | (hole4(q0.w) << 12) | (hole4(q1.x) << 16) |
-                 (hole4(q1.y) << 20) | (hole4(q1.z) << 24) | (hole4(q1.w) << 28);
-        } else {
-            for (int c = 0; c < BIN && x0 + c < F.W; c++)
-                if (__ldg(&row[c]) == 1) hm |= 1u << c;
-        }
-    }
-    if (!__syncthreads_or(hm != 0u)) return;  // CTA-uniform
-
-    const int cnt = __ldcg(&F.bin_count[b]);
-    const bool overflow = cnt > BIN_CAP;
-    const int nloc = overflow ? 0 : cnt;
-    for (int s = threadIdx.x; s < nloc; s += blockDim.x) {
-        const int i = __ldcg(&F.bin_list[(size_t)b * BIN_CAP + s]);
-        const float2 A = __ldg(&F.pts[i]), B = __ldg(&F.pts[i + 1]);
-        const float vx = __fsub_rn(B.x, A.x), vy = __fsub_rn(B.y, A.y);
-        const float l2 = __fadd_rn(__fmul_rn(vx, vx), __fmul_rn(vy, vy));
-        sg.av[s] = make_float4(A.x, A.y, vx, vy);
-        sg.inv_l2[s] = __fdiv_rn(1.0f, l2);
-        sg.id[s] = i;
-    }
-    // compact the hole pixels (row-major): row r's pixels follow rows 0..r-1
-    const int c = __popc(hm);  // 0 on lanes >= 4
-    int incl = c;
+            const unsigned km = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                const int pos = __popc(km & ((1u << lane) - 1u));
+                gw->av[pos] = S0;
+                gw->ilid[pos] = make_float2(__ldg(&F.segp[i].il32), __int_as_float(i));
+            }
+            __syncwarp();
+            const int m = __popc(km);
+            for (int s = 0; s < m; s++) {
+                const float4 S = gw->av[s];
+                const float2 t = gw->ilid[s];
+                const int id = __float_as_int(t.y);
 #pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 3) wtot[warp] = incl;
-    __syncthreads();
-    int base = 0, nh = 0;
-#pragma unroll
-    for (int w = 0; w < 8; w++) {
-        const int v = wtot[w];
-        if (w < warp) base += v;
-        nh += v;
-    }
-    if (lane < 4) {
-        int pos = base + incl - c;
-        for (uint32_t m = hm; m; m &= m - 1u) holes_s[pos++] = (short)((r << 5) | (__ffs(m) - 1));
-    }
-    __syncthreads();
-
-    float best[4];
-    int bi[4];
-    if (!overflow) {
-        if (nh <= 256) nearest_in_bin<1>(sg, nloc, holes_s, nh, x0, y0, best, bi);
-        else if (nh <= 512) nearest_in_bin<2>(sg, nloc, holes_s, nh, x0, y0, best, bi);
-        else nearest_in_bin<4>(sg, nloc, holes_s, nh, x0, y0, best, bi);
-    }
-    const float t3 = 3.0f * a.eta;
-    const float thr = __fmul_rn(t3, t3);
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-        const int q = threadIdx.x + 256 * j;
-        if (q >= nh) break;
-        const int e = holes_s[q];
-        const int x = x0 + (e & (BIN - 1)), y = y0 + (e >> 5);
-        float bd = best[j];
-        int bs = bi[j];
-        if (overflow) {
-            // the bin's list overflowed: every segment of the frame
-            bd = INFINITY;
-            bs = 0x7fffffff;
-            const float px = (float)x, py = (float)y;
-            for (int sp = 0; sp < F.n_splines; sp++) {
-                const int i0 = max(0, __ldg(&F.offsets[sp])), i1 = min(F.n_points, __ldg(&F.offsets[sp + 1]));
-                for (int i = i0; i + 1 < i1; i++) {
-                    const float2 A = __ldg(&F.pts[i]), B = __ldg(&F.pts[i + 1]);
-                    const float vx = __fsub_rn(B.x, A.x), vy = __fsub_rn(B.y, A.y);
-                    const float l2 = __fadd_rn(__fmul_rn(vx, vx), __fmul_rn(vy, vy));
-                    if (!(l2 > 0.0f)) continue;
-                    const float d2 = seg_d2(px, py, A.x, A.y, vx, vy, __fdiv_rn(1.0f, l2));
-                    if (d2 < bd || (d2 == bd && i < bs)) {
-                        bd = d2;
-                        bs = i;
+                for (int j = 0; j < P; j++) {
+                    const float d2 = seg_d2(px[j], py[j], S.x, S.y, S.z, S.w, t.x);
+                    if (d2 < best[j] || (d2 == best[j] && id < bi[j])) {
+                        best[j] = d2;
+                        bi[j] = id;
                     }
                 }
             }
         }
-        float2 out = make_float2(0.0f, 0.0f);
-        if (bs != 0x7fffffff && bd <= thr) {
-            // t = ((x - a).v) / |v|^2 clamped, d^2 = |x - a - t v|^2, g = (v/|v|) e^(-d^2/(2 eta^2)),
-            // with the reciprocals 1/|v|^2 and 1/(2 eta^2) precomputed in FP64
-            const double *s = F.seg64 + 8 * (size_t)bs;
-            const double ax = __ldcg(&s[0]), ay = __ldcg(&s[1]), vx = __ldcg(&s[2]), vy = __ldcg(&s[3]);
-            const double inv_l2 = __ldcg(&s[4]), tx = __ldcg(&s[5]), ty = __ldcg(&s[6]), sw = __ldcg(&s[7]);
-            const double wx = __dsub_rn((double)x, ax), wy = __dsub_rn((double)y, ay);
-            double t = __dmul_rn(__dadd_rn(__dmul_rn(wx, vx), __dmul_rn(wy, vy)), inv_l2);
-            if (t < 0.0) t = 0.0;
-            if (t > 1.0) t = 1.0;
-            const double qx = __dsub_rn(wx, __dmul_rn(t, vx)), qy = __dsub_rn(wy, __dmul_rn(t, vy));
-            const double d2 = __dadd_rn(__dmul_rn(qx, qx), __dmul_rn(qy, qy));
-            const double ev = exp(-__dmul_rn(d2, a.k2));
-            out.x = (float)__dmul_rn(__dmul_rn(tx, ev), sw);
-            out.y = (float)__dmul_rn(__dmul_rn(ty, ev), sw);
+    } else {
+        // the bin's list overflowed: every segment of the frame
+        for (int sp = 0; sp < F.n_splines; sp++) {
+            const int i0 = max(0, __ldg(&F.offsets[sp])), i1 = min(F.n_points, __ldg(&F.offsets[sp + 1]));
+            for (int i = i0; i + 1 < i1; i++) {
+                const float2 A = __ldg(&F.pts[i]), B = __ldg(&F.pts[i + 1]);
+                const float vx = __fsub_rn(B.x, A.x), vy = __fsub_rn(B.y, A.y);
+                const float l2 = __fadd_rn(__fmul_rn(vx, vx), __fmul_rn(vy, vy));
+                if (!(l2 > 0.0f)) continue;
+                const float il = __fdiv_rn(1.0f, l2);
+#pragma unroll
+                for (int j = 0; j < P; j++) {
+                    const float d2 = seg_d2(px[j], py[j], A.x, A.y, vx, vy, il);
+                    if (d2 < best[j] || (d2 == best[j] && i < bi[j])) {
+                        best[j] = d2;
+                        bi[j] = i;
+                    }
+                }
+            }
         }
-        F.guide[(size_t)y * F.W + x] = out;
     }
+    const float t3 = 3.0f * a.eta;
+    const float thr = __fmul_rn(t3, t3);
+#pragma unroll
+    for (int j = 0; j < P; j++)
+        if (lane + 32 * j < nh)
+            gw->seg[lane + 32 * j] = bi[j] != 0x7fffffff && best[j] <= thr ? bi[j] : -1;
 }
 
-// The weight of the spline holding each segment, for the frames of one chunk
-// that have weights: one CTA per frame, after bin_kernel.
-__global__ void __launch_bounds__(256) spline_weight_kernel(const __grid_constant__ GuideArgs a,
-                                                            const __grid_constant__ WeightChunk c)
+// One CTA per eight bins, in 32 strips of STRIP rows.  Lane 8 c + r of a warp reads row r
+// of a strip (two 16-byte loads where the row is aligned and inside the frame) into a
+// 32-bit hole mask; a CTA without hole pixels, most of them, ends there.  The strips with
+// hole pixels are then taken by the warps one at a time (dense strips cost several times
+// sparse ones).  The value is evaluated in one place: unrolled per pixel, it made the
+// kernel wait for instructions 40 % of the time.
+__global__ void __launch_bounds__(32 * GUIDE_WARPS, 4) guide_kernel(const __grid_constant__ GuideArgs a)
 {
-    const float *w = c.w[blockIdx.x];
-    if (!w) return;
-    const SplineFrameDev &F = a.frames[c.first + blockIdx.x];
-    for (int i = threadIdx.x; i + 1 < F.n_points; i += blockDim.x) {
-        int lo = 0, hi = F.n_splines;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (__ldg(&F.offsets[mid]) <= i) lo = mid; else hi = mid;
+    constexpr int PER = BIN / STRIP;                 // strips of a bin
+    constexpr int ITEMS = 4 * GUIDE_WARPS;           // strips of a CTA
+    constexpr int BINS = ITEMS / PER;
+    __shared__ GuideWarp s_warp[GUIDE_WARPS];
+    __shared__ uint32_t s_mask[ITEMS][STRIP];
+    __shared__ int s_frame[ITEMS];
+    __shared__ short s_list[ITEMS];
+    __shared__ int s_n, s_next;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) s_n = s_next = 0;
+    __syncthreads();
+    {
+        const int item = warp * 4 + (lane >> 3);     // strip item / BINS of bin item % BINS
+        const int gb = blockIdx.x * BINS + item % BINS;
+        uint32_t hm = 0u;
+        int f = 0;
+        if (gb < a.total_bins) {
+            f = find_frame(a.bin_offset, a.n_frames, gb);
+            const SplineFrameDev &F = a.frames[f];
+            const int b = gb - __ldg(&a.bin_offset[f]);
+            const int W = F.W, bx = b % F.NBX, by = b / F.NBX;
+            const int x0 = bx * BIN, y = by * BIN + item / BINS * STRIP + (lane & 7);
+            if (y < F.H) {
+                const uint8_t *row = F.labels + (size_t)y * W + x0;
+                if (x0 + BIN <= W && (reinterpret_cast<uintptr_t>(row) & 15u) == 0) {
+                    const uint4 q0 = __ldg(reinterpret_cast<const uint4 *>(row));
+                    const uint4 q1 = __ldg(reinterpret_cast<const uint4 *>(row) + 1);
+                    hm = hole4(q0.x) | (hole4(q0.y) << 4) | (hole4(q0.z) << 8) | (hole4(q0.w) << 12) |
+                         (hole4(q1.x) << 16) | (hole4(q1.y) << 20) | (hole4(q1.z) << 24) | (hole4(q1.w) << 28);
+                } else {
+                    for (int c = 0; c < BIN && x0 + c < W; c++)
+                        if (__ldg(&row[c]) == 1) hm |= 1u << c;
+                }
+            }
         }
-        if (F.n_splines <= 0 || i < __ldg(&F.offsets[0]) || i + 1 >= __ldg(&F.offsets[lo + 1])) continue;
-        F.seg64[8 * (size_t)i + 7] = (double)__ldg(&w[lo]);
+        const unsigned some = __ballot_sync(0xffffffffu, hm != 0u) & (0xffu << (lane & 24));
+        if (some) {
+            s_mask[item][lane & 7] = hm;
+            if ((lane & 7) == 0) {
+                s_frame[item] = f;
+                s_list[atomicAdd(&s_n, 1)] = (short)item;
+            }
+        }
+    }
+    __syncthreads();
+    const int n = s_n;
+    GuideWarp *gw = &s_warp[warp];
+    for (;;) {
+        int it = 0;
+        if (lane == 0) it = n > 0 ? atomicAdd(&s_next, 1) : n;
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= n) break;
+        const int item = s_list[it];
+        const int f = s_frame[item];
+        const SplineFrameDev &F = a.frames[f];
+        const int b = blockIdx.x * BINS + item % BINS - __ldg(&a.bin_offset[f]);
+        const int x0 = b % F.NBX * BIN, y0 = b / F.NBX * BIN + item / BINS * STRIP;
+        const int cnt = __ldg(&F.bin_count[b]);
+        // the hole pixels, row-major: lane l tests column l of each row
+        int nh = 0;
+        uint32_t cols = 0, rows = 0;
+#pragma unroll
+        for (int r = 0; r < STRIP; r++) {
+            const uint32_t m = s_mask[item][r];
+            cols |= m;
+            rows |= m ? 1u << r : 0u;
+            if ((m >> lane) & 1u) gw->holes[nh + __popc(m & ((1u << lane) - 1u))] = (short)((r << 5) | lane);
+            nh += __popc(m);
+        }
+        __syncwarp();
+        const float grow = 3.0f * a.eta + 1.0f;
+        const float4 box = make_float4((float)(x0 + __ffs(cols) - 1) - grow, (float)(x0 + 31 - __clz(cols)) + grow,
+                                       (float)(y0 + __ffs(rows) - 1) - grow, (float)(y0 + 31 - __clz(rows)) + grow);
+        if (nh <= 32) nearest_segments<1>(a, F, gw, b, cnt, x0, y0, nh, box);
+        else if (nh <= 64) nearest_segments<2>(a, F, gw, b, cnt, x0, y0, nh, box);
+        else if (nh <= 128) nearest_segments<4>(a, F, gw, b, cnt, x0, y0, nh, box);
+        else nearest_segments<8>(a, F, gw, b, cnt, x0, y0, nh, box);
+#pragma unroll 1
+        for (int q = lane; q < nh; q += 32) {
+            const int e = gw->holes[q], sgi = gw->seg[q];
+            const int x = x0 + (e & (BIN - 1)), y = y0 + (e >> 5);
+            float2 out = make_float2(0.0f, 0.0f);
+            if (sgi >= 0) {
+                SegPair sp;
+                const float4 *d = reinterpret_cast<const float4 *>(F.segp + sgi);
+                float4 *o = reinterpret_cast<float4 *>(&sp);
+#pragma unroll
+                for (int i = 0; i < 4; i++) o[i] = __ldg(&d[i]);
+                // coordinates that FP32 does not hold go the FP64 way
+                const bool sure = max(x, y) < (1 << 24) &&
+                                  guide_value((float)x, (float)y, sp, a.k2p, a.ieta, *a.exps, out.x, out.y);
+                if (!sure) out = guide_value64(F.seg64 + 8 * (size_t)sgi, x, y, a.k2);
+            }
+            F.guide[(size_t)y * F.W + x] = out;
+        }
+        __syncwarp();  // the strip's pixels have been read
     }
 }
 

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "../../include/guidefill.h"
+#include "gf_guide_math.cuh"
 
 namespace gf {
 
@@ -184,7 +185,9 @@ struct SplineFrameDev {
     float2 *guide;
     int32_t *bin_count;  // [NBX*NBY]
     int32_t *bin_list;   // [NBX*NBY*BIN_CAP]
-    double *seg64;       // [n_points][8]: per segment start a, v = b - a, 1/(|v|*|v|), v/|v| (FP64)
+    double *seg64;       // [n_points][8]: per segment start a, v = b - a, 1/(|v|*|v|), v/|v| (FP64), weight
+    SegPair *segp;       // [n_points]: the same as pairs of FP32 numbers
+    const float *weight; // [n_splines] or null (1)
 };
 
 struct GuideArgs {
@@ -195,6 +198,9 @@ struct GuideArgs {
     int32_t total_bins;
     float eta;
     double k2;                    // 1 / (2 eta^2) in FP64
+    Pair k2p;                     // the same as a pair
+    float ieta;                   // 1 / eta
+    const GuideExp *exps;         // written by upload_splines_kernel
 };
 
 constexpr int DESC_CHUNK = 128;  // frame descriptors per upload kernel
@@ -256,6 +262,7 @@ struct FrameChunk {
 struct SplineChunk {
     SplineFrameDev *dst_frames;
     int32_t *dst_po, *dst_bo;
+    GuideExp *dst_exps;
     int32_t first, count, last_chunk, pad;
     SplineFrameDev frames[DESC_CHUNK];
     int32_t po[DESC_CHUNK + 1];
