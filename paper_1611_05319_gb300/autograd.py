@@ -17,16 +17,28 @@ import torch
 from . import context
 
 
+_ONE_FIELD = 2 ** 31 - 64  # pixels that one guide field can have
+
+
 class GuidefillFunction(torch.autograd.Function):
     @staticmethod
     def forward(ctx, rgba, labels, mag, phi, mu, eps, c):
         g = context(rgba.device.index)
         B = rgba.shape[0]
         muf = float(mu)
-        guides = [g.guide_from_angle(labels[i], mag[i], phi[i]) for i in range(B)]
-        res = g.fill_batched([rgba[i] for i in range(B)], [labels[i] for i in range(B)], guides, eps=eps, mu=muf,
-                             c=c, stall=True)
-        out = torch.stack([r.rgba for r in res])
+        if 0 < labels.numel() <= _ONE_FIELD and labels.shape == mag.shape == phi.shape:
+            # one field B times as high: the conversion is per pixel
+            H, W = labels.shape[1:]
+            field = g.guide_from_angle(labels.reshape(B * H, W), mag.reshape(B * H, W), phi.reshape(B * H, W))
+            guides = list(field.view(B, H, W, 2).unbind())
+        else:
+            guides = [g.guide_from_angle(labels[i], mag[i], phi[i]) for i in range(B)]
+        # the frames' results are kept for the backward pass; the caller gets a copy to do
+        # with as it likes
+        kept = torch.empty(tuple(rgba.shape[:3]) + (4,), dtype=torch.float32, device=rgba.device)
+        res = g.fill_batched(list(rgba.unbind()), list(labels.unbind()), guides, eps=eps, mu=muf, c=c,
+                             out=list(kept.unbind()), stall=True)
+        out = kept.clone()
         ctx.res = res
         ctx.guides = guides
         ctx.eps, ctx.mu, ctx.c = eps, muf, c
@@ -37,10 +49,12 @@ class GuidefillFunction(torch.autograd.Function):
     def backward(ctx, grad_out):
         g = context(grad_out.device.index)
         B = grad_out.shape[0]
-        gi, gp, gmu = g.fill_backward(ctx.res, ctx.guides, [grad_out[i] for i in range(B)], eps=ctx.eps,
-                                      mu=ctx.mu, c=ctx.c)
-        grad_rgba = torch.stack(gi)
-        grad_phi = torch.stack(gp)
+        grad_out = grad_out.contiguous()
+        H, W = ctx.res[0].shell.shape
+        grad_rgba = torch.empty((B, H, W, 4), dtype=torch.float32, device=grad_out.device)
+        grad_phi = torch.empty((B, H, W), dtype=torch.float32, device=grad_out.device)
+        _, _, gmu = g.fill_backward(ctx.res, ctx.guides, list(grad_out.unbind()), eps=ctx.eps, mu=ctx.mu, c=ctx.c,
+                                    out=(grad_rgba.unbind(), grad_phi.unbind()))
         grad_mu = gmu.sum()
         if ctx.mu_device is not None:
             grad_mu = grad_mu.to(ctx.mu_device)
