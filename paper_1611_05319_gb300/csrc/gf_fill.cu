@@ -493,8 +493,9 @@ __device__ __forceinline__ unsigned long long around(const WarpSmem<RW> *ws, int
     return (unsigned long long)hi << 32 | lo;
 }
 
-// The rotated ball of one pixel, over the mirror pairs j, j + G, ...: readable
-// weights (unnormalised), whether any sample is readable, weighted colours.
+// The rotated ball of one pixel, over the mirror pairs j, j + G, ...: readable weights
+// (from the group weights eg), weighted colours, and the smallest |m| of a readable
+// sample, MAX_R + 1 when there is none.
 //
 // Negation is exact and commutes with every rounding of the rotation and of the
 // snap, so the second sample's offset is the exact negative of the first's; the
@@ -516,7 +517,7 @@ __device__ __forceinline__ unsigned long long around(const WarpSmem<RW> *ws, int
 // pixels 8,200 -> 6,100, 17 and more 13,100 -> 8,900, an iteration 620 -> 450.
 template <int RW, bool BITS>
 __device__ __forceinline__ void rotated_pairs(const FillParams &p, const WarpSmem<RW> *ws, const float *eg, int pix, int j,
-                                              int G, float ch, float sh, bool &any_, Acc &acc_)
+                                              int G, float ch, float sh, int &least_, Acc &acc_)
 {
     constexpr int WS = WarpSmem<RW>::WS, ZI = WS * WS;
     const int px = pix & 7, py = pix >> 3;
@@ -532,13 +533,14 @@ __device__ __forceinline__ void rotated_pairs(const FillParams &p, const WarpSme
         near = around<RW>(ws, px, py);
         rnear = __brevll(near);
     }
-    bool any = false;
+    int least = MAX_R + 1;
     Acc acc = {0ull, 0ull, 0.f, 0.f};
 #pragma unroll 1
     for (int q = j; q < npair; q += G) {
         const ulonglong2 nm = *reinterpret_cast<const ulonglong2 *>(&g_pos[q]);  // (n, n), (m, m)
         const float2 wt = g_wt[q];
-        const float w0 = eg[__float_as_int(wt.y) & 0xff] * wt.x;
+        const int gm = __float_as_int(wt.y) & 0xff;  // |m|
+        const float w0 = eg[gm] * wt.x;
         const unsigned long long o = add2(mul2(nm.x, c1), mul2(nm.y, c2));  // n ch - m sh, n sh + m ch
         const unsigned long long t = add2(o, big);
         const float2 d = unpack2(fma2(add2(t, nbig), neg1, o));             // o - rint(o), exact
@@ -564,7 +566,7 @@ __device__ __forceinline__ void rotated_pairs(const FillParams &p, const WarpSme
             ok1 = ((m1 >> (cx + fx)) & need) == need;
             ok2 = ((m2 >> (cx - fx - (hx ? 1 : 0))) & need) == need;
         }
-        any = any || ok1 || ok2;
+        if (ok1 || ok2) least = min(least, gm);
         weight_add(acc.s, acc.lo, (ok1 ? w0 : 0.f) + (ok2 ? w0 : 0.f));  // 0, w0 or 2 w0: exact
         const float gx = 1.f - frx;
         const float2 wy = unpack2(mul2(pack2(w0, w0), pack2(1.f - fry, fry)));
@@ -592,7 +594,7 @@ __device__ __forceinline__ void rotated_pairs(const FillParams &p, const WarpSme
         acc_add(acc, l, a3);
         acc_add(acc, l, b3);
     }
-    any_ = any;
+    least_ = least;
     acc_ = acc;
 }
 
@@ -602,15 +604,15 @@ __device__ __forceinline__ void rotated_pairs(const FillParams &p, const WarpSme
 // no exponential per sample to rescale them: a tile with 9 to 16 front pixels at eps
 // 5 takes 5,800 cycles instead of 20,400 (a 1500 x 1125 still 2.80 -> 0.96 ms with the
 // rest of this kernel).
-template <int RW, bool ISO>
+template <int RW, bool ISO, bool LEAST>
 __device__ __forceinline__ void lattice_pairs(const FillParams &p, const WarpSmem<RW> *ws, int pix, int j, int G, float2 g,
-                                              float &S_all_, bool &any_, Acc &acc_)
+                                              float &S_all_, bool &any_, Acc &acc_, float low, float &least_)
 {
     constexpr int WS = WarpSmem<RW>::WS, ZI = WS * WS;
     const ulonglong2 *col = reinterpret_cast<const ulonglong2 *>(ws->col);
     const int cx = (pix & 7) + RW, cy = (pix >> 3) + RW, c0 = cy * WS + cx;
     const int npair = p.tab.ns >> 1;
-    float S_all = 0.f;
+    float S_all = 0.f, least = INFINITY;
     bool any = false;
     Acc acc = {0ull, 0ull, 0.f, 0.f};
 #pragma unroll 2
@@ -618,14 +620,18 @@ __device__ __forceinline__ void lattice_pairs(const FillParams &p, const WarpSme
         const float2 wt = g_wt[q];
         const int code = __float_as_int(wt.y);
         const int n = ((code >> 8) & 0xff) - 8, m = ((code >> 16) & 0xff) - 8;
-        float w0 = wt.x;
+        float w0 = wt.x, e = 0.f;
         if (!ISO) {
             const float proj = -g.y * (float)n + g.x * (float)m;  // g_perp . (n, m)
-            w0 *= expf(-(p.coef32 * proj * proj));
+            const float t = p.coef32 * proj * proj;
+            // relative to `low`: exponents below it are those of samples that are not readable
+            w0 *= LEAST ? expf(low - (low > t ? low : t)) : expf(-t);
+            e = t;
         }
         const bool ok1 = (ws->rowmask[cy + m] >> (cx + n)) & 1u;
         const bool ok2 = (ws->rowmask[cy - m] >> (cx - n)) & 1u;
         any = any || ok1 || ok2;
+        if (LEAST && (ok1 || ok2)) least = fminf(least, e);
         S_all += w0 + w0;
         weight_add(acc.s, acc.lo, (ok1 ? w0 : 0.f) + (ok2 ? w0 : 0.f));
         const int at = m * WS + n;
@@ -635,50 +641,46 @@ __device__ __forceinline__ void lattice_pairs(const FillParams &p, const WarpSme
     }
     S_all_ = S_all;
     any_ = any;
+    if (LEAST) least_ = least;
     acc_ = acc;
 }
 
 struct PixelSums {
-    float S_rd, S_all, wsum;
+    float S_rd, S_all, wsum, lo;
     int cnt;
     float4 acc;
 };
 
 // One front pixel by the whole warp, each lane's colour sum relative to the smallest
 // weight exponent it has read (the normalisation cancels in the average and keeps
-// e^-t from underflowing): the pixels whose plain sums FP32 does not hold.  Must be
-// called by all 32 lanes; every lane gets the result.
+// e^-t from underflowing): rotated balls whose rotation is not one.  Must be called by
+// all 32 lanes; every lane gets the result.
 template <int RW>
-__device__ __noinline__ PixelSums slow_pixel(const FillParams &p, const WarpSmem<RW> *ws, int pix, bool ghost)
+__device__ __noinline__ PixelSums slow_pixel(const FillParams &p, const WarpSmem<RW> *ws, int pix)
 {
     constexpr int WS = WarpSmem<RW>::WS;
     const int lane = threadIdx.x & 31;
     const int px = pix & 7, py = pix >> 3;
     const float2 g = ws->guide[pix];
-    float ch = 1.0f, sh = 0.0f, beta = 0.0f;
-    if (ghost) {
-        const float a2 = __fadd_rn(__fmul_rn(g.x, g.x), __fmul_rn(g.y, g.y));
-        const float a = __fsqrt_rn(a2);
-        if (a > 0.0f) {
-            ch = __fdiv_rn(g.x, a);
-            sh = __fdiv_rn(g.y, a);
-        }
-        beta = p.coef32 * a2;
+    float ch = 1.0f, sh = 0.0f;
+    const float a2 = __fadd_rn(__fmul_rn(g.x, g.x), __fmul_rn(g.y, g.y));
+    const float a = __fsqrt_rn(a2);
+    if (a > 0.0f) {
+        ch = __fdiv_rn(g.x, a);
+        sh = __fdiv_rn(g.y, a);
     }
+    const float beta = p.coef32 * a2;
     float S_rd = 0.f, S_all = 0.f, tmin = INFINITY, wsum = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     int cnt = 0;
     for (int s = lane; s < p.tab.ns; s += 32) {
         const float nf = p.tab.n_f[s], mf = p.tab.m_f[s], invd = p.tab.invd[s];
-        float ox = nf, oy = mf;
-        if (ghost) {
-            ox = __fsub_rn(__fmul_rn(nf, ch), __fmul_rn(mf, sh));
-            oy = __fadd_rn(__fmul_rn(nf, sh), __fmul_rn(mf, ch));
-            float r0 = rintf(ox);
-            if (fabsf(__fsub_rn(ox, r0)) <= p.tau) ox = r0;
-            r0 = rintf(oy);
-            if (fabsf(__fsub_rn(oy, r0)) <= p.tau) oy = r0;
-        }
+        float ox = __fsub_rn(__fmul_rn(nf, ch), __fmul_rn(mf, sh));
+        float oy = __fadd_rn(__fmul_rn(nf, sh), __fmul_rn(mf, ch));
+        float r0 = rintf(ox);
+        if (fabsf(__fsub_rn(ox, r0)) <= p.tau) ox = r0;
+        r0 = rintf(oy);
+        if (fabsf(__fsub_rn(oy, r0)) <= p.tau) oy = r0;
         const float flx = floorf(ox), fly = floorf(oy);
         const float frx = __fsub_rn(ox, flx), fry = __fsub_rn(oy, fly);
         const int ix = px + RW + (int)flx, iy = py + RW + (int)fly;
@@ -687,13 +689,7 @@ __device__ __noinline__ PixelSums slow_pixel(const FillParams &p, const WarpSmem
         bool ok = ix >= 0 && iy >= 0 && ix < WS - 1 && iy < WS - 1;
         ok = ok && ((ws->rowmask[iy] >> ix) & need) == need;
         if (fry > 0.0f) ok = ok && (((ws->rowmask[iy + 1] >> ix) & need) == need);
-        float tt;
-        if (ghost) {
-            tt = beta * (mf * mf);
-        } else {
-            const float proj = -g.y * nf + g.x * mf;  // lattice ball: g_perp . (n, m)
-            tt = p.coef32 * proj * proj;
-        }
+        const float tt = beta * (mf * mf);
         S_all += expf(-tt) * invd;
         if (ok) {
             S_rd += expf(-tt) * invd;
@@ -732,7 +728,7 @@ __device__ __noinline__ PixelSums slow_pixel(const FillParams &p, const WarpSmem
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) tg = fminf(tg, __shfl_xor_sync(FULL, tg, o));
     const float sc = (tmin == INFINITY) ? 0.f : expf(tg - tmin);
-    PixelSums r = {S_rd, S_all, wsum * sc, cnt, make_float4(acc.x * sc, acc.y * sc, acc.z * sc, acc.w * sc)};
+    PixelSums r = {S_rd, S_all, wsum * sc, 0.f, cnt, make_float4(acc.x * sc, acc.y * sc, acc.z * sc, acc.w * sc)};
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         r.S_rd += __shfl_xor_sync(FULL, r.S_rd, o);
@@ -745,6 +741,68 @@ __device__ __noinline__ PixelSums slow_pixel(const FillParams &p, const WarpSmem
         r.acc.w += __shfl_xor_sync(FULL, r.acc.w, o);
     }
     return r;
+}
+
+// The colour and weight sums of the pixels of a pass (G lanes each) again, relative to
+// the smallest exponent of a readable sample: readable weights that all underflow in
+// FP32.  Without the ready test a pixel is filled whatever its weights are; with it a
+// rotated ball's ready pixels have S_rd > c S_all >= c times the m = 0 weights, but a
+// lattice ball's weights may all be tiny.  Out of line: rare, and inside the passes it
+// cost every tile 3 to 10 %; one pixel at a time it made onion-order fills with sharp
+// weights up to 1.7 times slower than now.  Must be called by all 32 lanes; `run`
+// marks the lanes of the pixels concerned, `least_m` is their smallest readable |m| (of
+// the rotated ball), and lane j = 0 of each gets the result.
+template <int RW>
+__device__ __noinline__ PixelSums redo_pixels(const FillParams &p, WarpSmem<RW> *ws, int pix, int grp, int j, int G,
+                                              bool run, bool ghost, int least_m)
+{
+    const float2 g = ws->guide[pix];
+    const int R = p.tab.R;
+    float ch = 1.0f, sh = 0.0f, beta = 0.0f;
+    if (ghost) {
+        const float a2 = __fadd_rn(__fmul_rn(g.x, g.x), __fmul_rn(g.y, g.y));
+        const float a = __fsqrt_rn(a2);
+        if (a > 0.0f) {
+            ch = __fdiv_rn(g.x, a);
+            sh = __fdiv_rn(g.y, a);
+        }
+        beta = p.coef32 * a2;
+    }
+    Acc acc = {0ull, 0ull, 0.f, 0.f};
+    if (ghost) {
+        __syncwarp();
+        if (run)
+            for (int gg = j; gg <= R; gg += G)
+                ws->eg[grp][gg] = gg < least_m ? 0.f : expf(-(beta * (float)(gg * gg - least_m * least_m)));
+        __syncwarp();
+        int unused;
+        if (run) rotated_pairs<RW, false>(p, ws, ws->eg[grp], pix, j, G, ch, sh, unused, acc);
+    } else {
+        float low = 0.f, least = INFINITY, all;  // exponents
+        bool any;
+        if (run) lattice_pairs<RW, false, true>(p, ws, pix, j, G, g, all, any, acc, low, least);
+        for (int o = 1; o < G; o <<= 1) {
+            const float l = __shfl_down_sync(FULL, least, o);
+            if (j + o < G) least = fminf(least, l);
+        }
+        low = __shfl_sync(FULL, least, threadIdx.x % 32 - j);
+        if (run) lattice_pairs<RW, false, true>(p, ws, pix, j, G, g, all, any, acc, low, least);
+    }
+    float2 axy = unpack2(acc.xy), azw = unpack2(acc.zw);
+    for (int o = 1; o < G; o <<= 1) {
+        const float s0 = __shfl_down_sync(FULL, acc.s, o), s1 = __shfl_down_sync(FULL, acc.lo, o);
+        const float c0 = __shfl_down_sync(FULL, axy.x, o), c1 = __shfl_down_sync(FULL, axy.y, o);
+        const float c2 = __shfl_down_sync(FULL, azw.x, o), c3 = __shfl_down_sync(FULL, azw.y, o);
+        if (j + o < G) {
+            weight_add(acc.s, acc.lo, s0);
+            acc.lo += s1;
+            axy.x += c0;
+            axy.y += c1;
+            azw.x += c2;
+            azw.y += c3;
+        }
+    }
+    return PixelSums{0.f, 0.f, acc.s, acc.lo, 0, make_float4(axy.x, axy.y, azw.x, azw.y)};
 }
 
 // The three work lists of a cluster (the list of step s in slot s % 3): the
@@ -1034,6 +1092,7 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
             if (act && MODE != STALL) g = ws->guide[pix];
             float S_all = 0.f;
             bool any = false, odd = false;
+            int least = MAX_R + 1;  // rotated ball: smallest |m| of a readable sample
             Acc acc = {0ull, 0ull, 0.f, 0.f};
             if (MODE != STALL && ghost) {
                 float ch = 1.0f, sh = 0.0f;
@@ -1056,13 +1115,15 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
                 __syncwarp();
                 if (act && !odd) {
                     const float *eg = ws->eg[grp];
-                    if (RW == 4 && p.tau >= 6e-6f) rotated_pairs<RW, true>(p, ws, eg, pix, j, G, ch, sh, any, acc);
-                    else rotated_pairs<RW, false>(p, ws, eg, pix, j, G, ch, sh, any, acc);
+                    if (RW == 4 && p.tau >= 6e-6f) rotated_pairs<RW, true>(p, ws, eg, pix, j, G, ch, sh, least, acc);
+                    else rotated_pairs<RW, false>(p, ws, eg, pix, j, G, ch, sh, least, acc);
+                    any = least <= R;
                     if (decide && j == 0)
                         for (int gg = 0; gg <= R; gg++) S_all = __fmaf_rn(eg[gg], p.tab.Dm[gg], S_all);
                 }
             } else if (act) {
-                lattice_pairs<RW, MODE == STALL>(p, ws, pix, j, G, g, S_all, any, acc);
+                float unused;
+                lattice_pairs<RW, MODE == STALL, false>(p, ws, pix, j, G, g, S_all, any, acc, 0.f, unused);
             }
             // combine the lanes of a pixel: lane j takes from j + 1, then j + 2, ...
             float2 axy = unpack2(acc.xy), azw = unpack2(acc.zw);
@@ -1081,32 +1142,43 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
                 if (!plain) {
                     const float a1 = __shfl_down_sync(FULL, S_all, o);
                     const bool an = __shfl_down_sync(FULL, (int)any, o) != 0;
+                    const int l1 = __shfl_down_sync(FULL, least, o);
                     if (in) {
                         S_all += a1;
                         any = any || an;
+                        least = min(least, l1);
                     }
                 }
             }
             if (plain) any = S_rd > 0.f;
-            // Sums that FP32 holds badly: readable weights that all underflow (without the
-            // ready test a pixel is filled whatever they are; with it a rotated ball's ready
-            // pixels have S_rd > c S_all >= c times the m = 0 weights, but a lattice ball's
-            // weights may all be tiny), and rotations that are not one.  Those pixels are
-            // done again, one at a time, relative to their smallest readable exponent.
             float wsum = S_rd;
-            const bool redo = act && j == 0 && MODE != STALL &&
-                              (odd || (any && !(decide ? ghost || S_all >= 1e-18f : !(S_rd < 1e-18f))));
-            for (unsigned rb = __ballot_sync(FULL, redo); rb; rb &= rb - 1u) {
-                const int src = __ffs(rb) - 1;
-                const PixelSums r = slow_pixel<RW>(p, ws, __shfl_sync(FULL, pix, src), ghost);
-                if (lane == src) {
-                    S_rd = r.S_rd;
-                    S_all = r.S_all;
-                    any = r.cnt > 0;
-                    axy = make_float2(r.acc.x, r.acc.y);
-                    azw = make_float2(r.acc.z, r.acc.w);
-                    wsum = r.wsum;
-                    S_lo = 0.f;
+            if (!plain) {
+                const bool redo = act && j == 0 && any && !odd && (decide ? S_all < 1e-18f : S_rd < 1e-18f);
+                if (__any_sync(FULL, redo)) {
+                    const bool mine = __shfl_sync(FULL, (int)redo, lane - j) != 0;
+                    const PixelSums r = redo_pixels<RW>(p, ws, pix, grp, j, G, mine, ghost, __shfl_sync(FULL, least, lane - j));
+                    if (redo) {
+                        axy = make_float2(r.acc.x, r.acc.y);
+                        azw = make_float2(r.acc.z, r.acc.w);
+                        wsum = r.wsum;
+                        S_lo = r.lo;
+                    }
+                }
+            }
+            // rotations that are not one: the general way, one pixel at a time
+            if (MODE != STALL && ghost) {
+                for (unsigned rb = __ballot_sync(FULL, act && j == 0 && odd); rb; rb &= rb - 1u) {
+                    const int src = __ffs(rb) - 1;
+                    const PixelSums r = slow_pixel<RW>(p, ws, __shfl_sync(FULL, pix, src));
+                    if (lane == src) {
+                        S_rd = r.S_rd;
+                        S_all = r.S_all;
+                        any = r.cnt > 0;
+                        axy = make_float2(r.acc.x, r.acc.y);
+                        azw = make_float2(r.acc.z, r.acc.w);
+                        wsum = r.wsum;
+                        S_lo = 0.f;
+                    }
                 }
             }
             // Smart order: decided in FP32 outside a guard band around c, re-checked in
