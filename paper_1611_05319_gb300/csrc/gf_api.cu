@@ -1070,7 +1070,7 @@ gf_status gf_detect_splines_batched(gf_ctx *ctx, int n, const gf_detect_frame *f
     // scratch per frame: distances, tile flags, edge classes, union-find, candidates, row-segment masks
     std::vector<DetectFrameDev> hd(n);
     std::vector<int32_t> hto(n + 1);
-    std::vector<size_t> o_mask(n), o_dist(n), o_edge(n), o_par(n), o_mark(n), o_cand(n), o_accm(n), o_accp(n);
+    std::vector<size_t> o_mask(n), o_dist(n), o_edge(n), o_par(n), o_mark(n), o_cand(n), o_accm(n), o_row(n);
     std::vector<int32_t> hwo(n + 1);
     int64_t words = 0;
     size_t pos = 0;
@@ -1086,7 +1086,6 @@ gf_status gf_detect_splines_batched(gf_ctx *ctx, int n, const gf_detect_frame *f
         o_mark[i] = pos; pos = align_up(pos + 4 * np, 256);
         o_cand[i] = pos; pos = align_up(pos + 16 * np, 256);
         o_accm[i] = pos; pos = align_up(pos + 4 * (size_t)frames[i].H * NBX, 256);
-        o_accp[i] = pos; pos = align_up(pos + 4 * (size_t)frames[i].H * NBX, 256);
         hto[i] = (int32_t)tiles;
         tiles += (int64_t)NBX * NBY;
         hwo[i] = (int32_t)words;
@@ -1100,8 +1099,13 @@ gf_status gf_detect_splines_batched(gf_ctx *ctx, int n, const gf_detect_frame *f
     const size_t o_wo = pos; pos = align_up(pos + 4 * (size_t)(n + 1), 256);
     const size_t o_list = pos; pos = align_up(pos + 4 * (size_t)tiles, 256);
     const size_t o_slist = pos; pos = align_up(pos + 4 * (size_t)tiles, 256);
-    const size_t o_cnt = pos; pos = align_up(pos + 8, 256);                 // active, slow counts
-    const size_t o_flags = pos; pos = align_up(pos + 2 * (size_t)tiles, 256);  // hole_t, act_t (cleared)
+    // what starts at zero, in one piece: active and slow counts, hole_t and act_t, row counts
+    const size_t o_cnt = pos; pos = align_up(pos + 8, 256);
+    const size_t o_flags = pos; pos = align_up(pos + 2 * (size_t)tiles, 256);
+    for (int i = 0; i < n; i++) {
+        o_row[i] = pos; pos = align_up(pos + 4 * (size_t)frames[i].H, 256);
+    }
+    const size_t zero_end = pos;
     const size_t o_slow = pos; pos = align_up(pos + (size_t)tiles, 256);       // slow_t
     gf_status s = ensure(ctx, ctx->darena, pos);
     if (s != GF_OK) return s;
@@ -1123,7 +1127,7 @@ gf_status gf_detect_splines_batched(gf_ctx *ctx, int n, const gf_detect_frame *f
         d.mark = (int32_t *)(A + o_mark[i]);
         d.cand = (float4 *)(A + o_cand[i]);
         d.accm = (uint32_t *)(A + o_accm[i]);
-        d.accpos = (uint32_t *)(A + o_accp[i]);
+        d.row = (int32_t *)(A + o_row[i]);
         d.pts = (float2 *)f.pts; d.weight = f.weight; d.offsets = f.offsets; d.base = f.base;
         d.edges_out = f.edges; d.result = f.result;
         d.max_splines = f.max_splines;
@@ -1179,8 +1183,7 @@ gf_status gf_detect_splines_batched(gf_ctx *ctx, int n, const gf_detect_frame *f
     int per_sm_dist = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_dist, detect_dist_kernel, DET_THREADS, sm_dist));
     const unsigned g_dist = (unsigned)std::min<int64_t>(tiles, (int64_t)std::max(per_sm_dist, 1) * ctx->sm_count);
-    CK(cudaMemsetAsync(A + o_cnt, 0, 8, st));
-    CK(cudaMemsetAsync(A + o_flags, 0, 2 * (size_t)tiles, st));
+    CK(cudaMemsetAsync(A + o_cnt, 0, zero_end - o_cnt, st));
     for (int i = 0; i < n; i++)
         if (frames[i].edges) CK(cudaMemsetAsync(frames[i].edges, 0, (size_t)frames[i].H * frames[i].W, st));
     detect_pack_kernel<<<(unsigned)((words + 255) / 256), 256, 0, st>>>(da, (int)words);

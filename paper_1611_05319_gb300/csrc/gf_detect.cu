@@ -859,78 +859,56 @@ __global__ void __launch_bounds__(DET_THREADS) detect_accept_kernel(const __grid
             bool kept = false;
             if (e[j]) kept = __ldcg(&F.mark[uf_find(par, Y * F.W + X, budget)]) != 0;
             const uint32_t m = __ballot_sync(0xffffffffu, kept && ring[j]);
-            if (lane == 0) F.accm[(size_t)Y * F.NBX + d.tx] = m;
+            if (lane == 0) {
+                F.accm[(size_t)Y * F.NBX + d.tx] = m;
+                if (m) atomicAdd(&F.row[Y], __popc(m));
+            }
             if (F.edges_out && X < F.W) F.edges_out[(size_t)Y * F.W + X] = kept ? 1 : 0;
         }
         if (budget <= 0) atomicExch(&F.result[1], (int)GF_ERR_TIMEOUT);
     }
 }
 
-// One CTA per frame: output positions in raster order, the exclusive prefix of
-// the accepted counts over the frame's row segments [H][NBX].  Each warp takes a
-// contiguous run of segments, 32 consecutive ones per step (coalesced): first
-// the runs' totals, their prefix over the warps, then the positions.  Also the
-// count and the polyline offsets.
+// One CTA per frame: output positions in raster order, here of each row's first
+// accepted pixel (the exclusive prefix of the rows' counts); the write kernel adds the
+// segments before its own in the row, for the few segments that hold one.  (A prefix over
+// all row segments, 64,800 of a 1080p frame, took 72 us in one CTA; the rows' takes 4.)  Also the count and the polyline offsets.
 __global__ void __launch_bounds__(DET_SCAN_THREADS) detect_scan_kernel(const __grid_constant__ DetectArgs a)
 {
-    constexpr int NWARP = DET_SCAN_THREADS / 32;
-    __shared__ uint32_t wsum[NWARP];
-    __shared__ uint32_t total_s;
+    __shared__ int wsum[DET_SCAN_THREADS / 32];
+    __shared__ int carry_s;
     const DetectFrameDev &F = a.frames[blockIdx.x];
-    const int n = F.H * F.NBX;
+    const int H = F.H;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int per = (((n + NWARP - 1) / NWARP) + 31) & ~31;
-    const int s0 = min(n, warp * per), s1 = min(n, s0 + per);
-    // the accepted ring pixels of row segment i (Y = i / NBX, tile column i % NBX); 0 outside
-    // active tiles.  A warp's runs are read four steps of 32 at a time (independent loads).
-    auto seg_count = [&](int i) -> uint32_t {
-        if (i >= s1) return 0u;
-        const int Y = i / F.NBX, tx = i - Y * F.NBX;
-        const uint32_t m = __ldcg(&F.accm[i]);
-        return __ldcg(&F.act_t[(Y >> 5) * F.NBX + tx]) ? (uint32_t)__popc(m) : 0u;
-    };
-    uint32_t tot = 0;
-    for (int b = s0; b < s1; b += 128) {
-        uint32_t c4[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) c4[u] = seg_count(b + 32 * u + lane);
-#pragma unroll
-        for (int u = 0; u < 4; u++) tot += __reduce_add_sync(0xffffffffu, c4[u]);
-    }
-    if (lane == 0) wsum[warp] = tot;
-    __syncthreads();
-    if (warp == 0) {
-        const uint32_t v = wsum[lane];
-        uint32_t w = v;
+    int carry = 0;
+    for (int base = 0; base < H; base += DET_SCAN_THREADS) {
+        const int i = base + threadIdx.x;
+        const int v = i < H ? __ldcg(&F.row[i]) : 0;
+        int x = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += u;
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
         }
-        wsum[lane] = w - v;  // exclusive
-        if (lane == 31) total_s = w;
-    }
-    __syncthreads();
-    uint32_t run = wsum[warp];
-    for (int b = s0; b < s1; b += 128) {
-        uint32_t c4[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) c4[u] = seg_count(b + 32 * u + lane);
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const int i = b + 32 * u + lane;
-            const uint32_t c = c4[u];
-            uint32_t incl = c;
+        if (lane == 31) wsum[warp] = x;
+        __syncthreads();
+        if (warp == 0) {
+            int w = wsum[lane];
+            const int own = w;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t v2 = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v2;
+                const int y = __shfl_up_sync(0xffffffffu, w, o);
+                if (lane >= o) w += y;
             }
-            if (i < s1) F.accpos[i] = run + incl - c;
-            run += __shfl_sync(0xffffffffu, incl, 31);
+            wsum[lane] = w - own;
+            if (lane == 31) carry_s = w;
         }
+        __syncthreads();
+        if (i < H) F.row[i] = carry + wsum[warp] + x - v;
+        carry += carry_s;
+        __syncthreads();  // wsum and carry_s have been read
     }
-    const uint32_t total = total_s;
+    const uint32_t total = (uint32_t)carry;
     if (threadIdx.x == 0) F.result[0] = (int32_t)total;
     for (int k = threadIdx.x; k <= F.max_splines; k += DET_SCAN_THREADS)
         F.offsets[k] = 2 * (int32_t)min((uint32_t)k, total);
@@ -946,10 +924,15 @@ __global__ void __launch_bounds__(DET_THREADS) detect_write_kernel(const __grid_
         for (int rr = warp; rr < DT; rr += DET_THREADS / 32) {
             const int Y = d.y0 + rr, X = d.x0 + lane;
             if (Y >= F.H) break;
-            const size_t seg = (size_t)Y * F.NBX + d.tx;
-            const uint32_t m = F.accm[seg];
+            const uint32_t m = F.accm[(size_t)Y * F.NBX + d.tx];
+            if (m == 0u) continue;  // warp-uniform
+            // accepted pixels of the row's segments before this one (written in active tiles only)
+            int before = 0;
+            for (int t = lane; t < d.tx; t += 32)
+                if (__ldcg(&F.act_t[(Y >> 5) * F.NBX + t])) before += __popc(__ldcg(&F.accm[(size_t)Y * F.NBX + t]));
+            before = __reduce_add_sync(0xffffffffu, before);
             if (!((m >> lane) & 1u)) continue;
-            const uint32_t pos = F.accpos[seg] + __popc(m & ((1u << lane) - 1u));
+            const uint32_t pos = (uint32_t)(__ldcg(&F.row[Y]) + before) + __popc(m & ((1u << lane) - 1u));
             if (pos >= (uint32_t)F.max_splines) continue;
             const int p = Y * F.W + X;
             const float4 c = F.cand[p];

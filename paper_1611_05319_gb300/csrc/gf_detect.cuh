@@ -30,7 +30,8 @@ struct DetectFrameDev {
     int32_t *mark;        // [H][W] set at roots whose component holds a strong pixel
     float4 *cand;         // [H][W] at ring pixels on an edge: spline end x, end y, weight
     uint32_t *accm;       // [H][NBX] accepted ring pixels of each 32-pixel row segment (bit = column)
-    uint32_t *accpos;     // [H][NBX] output position of the segment's first accepted pixel
+    int32_t *row;         // [H] accepted ring pixels of the row (cleared; accept), then their output
+                          // position (scan)
     float2 *pts;          // [max_splines][2]
     float *weight;        // [max_splines]
     int32_t *offsets;     // [max_splines + 1]
