@@ -472,15 +472,16 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
         off_S[i] = pos; pos = align_up(pos + 4 * (size_t)ntiles[i], 256);
         off_L[i] = pos; pos = align_up(pos + 4 * (size_t)ntiles[i], 256);
     }
-    // what starts at zero, in one piece: hole counts, guided counts, front counts, teams
+    // what starts at zero, in one piece: hole counts, guided counts, front counts, teams,
+    // the queue heads, and for one frame its place in the order
     const size_t off_holes = pos; pos = align_up(pos + 4 * (size_t)n, 256);
     const size_t off_gleft = pos; pos = align_up(pos + 4 * (size_t)n, 256);
     const size_t off_icnt = pos; pos = align_up(pos + 8 * (size_t)n, 256);
     const size_t off_teams = pos; pos = align_up(pos + sizeof(TeamCtl) * (size_t)n, 256);
+    const size_t off_cursor = pos; pos = align_up(pos + 8, 256);  // queue heads of the two launches
+    const size_t off_order = pos; pos = align_up(pos + 4 * (size_t)n, 256);
     const size_t off_zero_end = pos;
     const size_t off_desc = pos; pos = align_up(pos + sizeof(FrameDev) * (size_t)n, 256);
-    const size_t off_order = pos; pos = align_up(pos + 4 * (size_t)n, 256);
-    const size_t off_cursor = pos; pos = align_up(pos + 8, 256);  // queue heads of the two launches
     const size_t off_ctaoff = pos; pos = align_up(pos + 4 * (size_t)(n + 1), 256);
 
     // ---- launch shape
@@ -562,6 +563,7 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
         int64_t cap = prm->max_shells > 0 ? std::min<int64_t>(prm->max_shells, full) : full;
         d.max_shells = (int32_t)std::min<int64_t>(cap, INT32_MAX - 2);
         d.rgba = (float4 *)f.out_rgba;
+        d.src = f.out_rgba != f.rgba ? (const float4 *)f.rgba : nullptr;
         d.labels = f.labels;
         d.guide = (const float2 *)f.guide;
         d.shell = f.out_shell;
@@ -578,7 +580,7 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
         d.init_count = (int32_t *)(A + off_icnt) + 2 * i;
         hd[i] = d;
         hcta[i] = (int32_t)ctas;
-        ctas += (int64_t)init_ctas(d.TH, f.W);
+        ctas += (int64_t)init_ctas(d.TH, f.W) + (d.src ? copy_ctas((int64_t)f.H * f.W) : 0);
     }
     hcta[n] = (int32_t)ctas;
     if (ctas >= INT32_MAX) return GF_ERR_ARG;
@@ -656,6 +658,8 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
             static thread_local FrameChunk ch;  // large: keep off the stack
             ch.dst_frames = (FrameDev *)(A + off_desc);
             ch.dst_cta = (int32_t *)(A + off_ctaoff);
+            ch.zero = (uint4 *)(A + off_holes);
+            ch.zero16 = c0 == 0 ? (int64_t)((off_zero_end - off_holes) / 16) : 0;
             ch.first = c0;
             ch.count = std::min(DESC_CHUNK, n - c0);
             ch.last_chunk = (c0 + ch.count == n) ? 1 : 0;
@@ -664,18 +668,8 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
                 ch.cta[i] = hcta[c0 + i];
             }
             ch.cta[ch.count] = hcta[c0 + ch.count];
-            upload_frames_kernel<<<1, 128, 0, stream>>>(ch);
+            upload_frames_kernel<<<1, 512, 0, stream>>>(ch);
             e = cudaGetLastError();
-        }
-        if (e) break;
-        e = cudaMemsetAsync(A + off_holes, 0, off_zero_end - off_holes, stream);
-        if (e) break;
-        for (int i = 0; i < n && !e; i++) {
-            const gf_frame &f = frames[i];
-            if (f.out_rgba != f.rgba)
-                e = cudaMemcpyAsync(f.out_rgba, f.rgba, (size_t)f.H * f.W * 16, cudaMemcpyDeviceToDevice, stream);
-            if (!e && f.out_stall)
-                e = cudaMemsetAsync(f.out_stall, 0, 4 * (((size_t)f.H * f.W + 1 + 31) / 32), stream);
         }
         if (e) break;
         InitArgs ia;
@@ -688,7 +682,7 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
             if (hcta[i + 1] - hcta[i] != ia.uniform_ctas) ia.uniform_ctas = 0;
         init_kernel<<<(unsigned)ctas, 32 * INIT_WARPS, 0, stream>>>(ia);
         e = cudaGetLastError();
-        if (e) break;
+        if (e || n == 1) break;
         order_kernel<<<1, 256, 0, stream>>>(fp.frames, n, fp.frame_order, fp.frame_cursor);
         e = cudaGetLastError();
     } while (0);

@@ -27,6 +27,10 @@ __host__ __device__ inline int init_ctas(int TH, int W) {
     const int strips = ((W + 7) / 8 + 31) / 32;
     return (TH * strips + INIT_WARPS - 1) / INIT_WARPS;
 }
+// and, when the output is another image than the input, CTAs that copy COPY_PIXELS
+// colours each
+constexpr int COPY_PIXELS = 32 * INIT_WARPS * 8;
+__host__ __device__ inline int64_t copy_ctas(int64_t px) { return (px + COPY_PIXELS - 1) / COPY_PIXELS; }
 
 // Per-pixel state word (out_shell): readable at step k  <=>  (uint)(s+1) < (uint)(k+1)
 constexpr int32_t SH_KNOWN = -1;
@@ -79,6 +83,7 @@ struct FrameDev {
     int32_t H, W, TW, TH, ntiles;
     int32_t max_shells;
     float4 *rgba;                 // working image (out_rgba)
+    const float4 *src;            // input image to copy there, or null
     const uint8_t *labels;
     const float2 *guide;
     int32_t *shell;
@@ -255,6 +260,8 @@ cudaError_t launch_adj(int rr, const cudaLaunchConfig_t &cfg, const AdjArgs &a);
 struct FrameChunk {
     FrameDev *dst_frames;
     int32_t *dst_cta;
+    uint4 *zero;                  // scratch that starts at zero, cleared with the first chunk (or null)
+    int64_t zero16;               // its length in 16-byte words
     int32_t first, count, last_chunk, pad;
     FrameDev frames[DESC_CHUNK];
     int32_t cta[DESC_CHUNK + 1];

@@ -199,6 +199,8 @@ extern "C" gf_status gf_fill_noalloc(const gf_frame *f, const gf_params *p, gf_s
     static thread_local FrameChunk ch;
     ch.dst_frames = (FrameDev *)(A + l.desc);
     ch.dst_cta = (int32_t *)(A + l.ctaoff);
+    ch.zero = nullptr;
+    ch.zero16 = 0;
     ch.first = 0;
     ch.count = 1;
     ch.last_chunk = 1;
