@@ -359,8 +359,9 @@ gf_status gf_fill_backward(gf_ctx *ctx, int n, const gf_adjoint_frame *frames, c
 /*
  * Launch shape of the persistent fill (no counterpart in the paper; a tuning
  * knob of this implementation).  cluster_size in {0 (automatic), 1, 2, 4, 8,
- * 16} CTAs per frame; n_clusters = number of persistent clusters (0 = as many
- * as fit, capped at the number of frames); use_graph = capture the batched
+ * 16} CTAs per cluster; n_clusters = number of persistent clusters (0 = as many
+ * as fit and the frames can use: clusters without a frame of their own join
+ * running frames, see gf_fill.cu); use_graph = capture the batched
  * launch sequence into a CUDA graph and replay it (streams other than the
  * legacy default stream only).  Results do not depend on the launch shape.
  */

@@ -872,7 +872,8 @@ __global__ void __launch_bounds__(DET_THREADS) detect_accept_kernel(const __grid
 // One CTA per frame: output positions in raster order, here of each row's first
 // accepted pixel (the exclusive prefix of the rows' counts); the write kernel adds the
 // segments before its own in the row, for the few segments that hold one.  (A prefix over
-// all row segments, 64,800 of a 1080p frame, took 72 us in one CTA; the rows' takes 4.)  Also the count and the polyline offsets.
+// all row segments, 64,800 of a 1080p frame, took 72 us in one CTA; the rows' takes 4.)
+// Also the count and the polyline offsets.
 __global__ void __launch_bounds__(DET_SCAN_THREADS) detect_scan_kernel(const __grid_constant__ DetectArgs a)
 {
     __shared__ int wsum[DET_SCAN_THREADS / 32];

@@ -1,7 +1,8 @@
 // Shell-by-shell transport fill (Guidefill, arxiv 1611.05319) for sm_103a.
 //
 // Kernels:
-//   init_kernel   one pass over every frame: state word per pixel (out_shell),
+//   init_kernel   one pass over every frame: the image copied to the output where
+//                 that is another, state word per pixel (out_shell),
 //                 per 8x8 tile the bitmask of hole pixels (U) and of the initial
 //                 active boundary (Qw = d_active D^(0)_h, Notation) from bit
 //                 operations on the labels, per-frame hole count.
@@ -10,7 +11,9 @@
 //                 with larger clusters, running beside the first).
 //   fill_kernel   persistent; one thread-block cluster runs one frame's whole
 //                 shell loop (Algorithm 1) at a time, with one hardware cluster
-//                 barrier per step, then takes the next frame from the queue.
+//                 barrier per step, then takes the next frame from the queue;
+//                 clusters that find the queue empty join running frames
+//                 (Teams, below).
 //
 // Front tracking.  Per step k the cluster processes a work list of tiles.  A
 // tile is on the list of step k+1 iff a pixel was filled at step k within
@@ -66,10 +69,6 @@ __shared__ float2 g_wt[MAX_SAMPLES / 2];
 // ---------------------------------------------------------------------------
 // init
 // ---------------------------------------------------------------------------
-// Also what a fill starts from: the copy of the input where the output is another image
-// (CTAs of their own) and the cleared stall bitmap.  With the scratch cleared by the
-// descriptor upload and no order kernel for one frame, a single fill is three launches
-// instead of six or seven: the 128 x 128 frame 107 -> 96 us a call.
 // One warp per strip of 8 pixel rows x 32 tiles (256 columns); lane l owns tile
 // column 32 s + l, i.e. 8 pixel columns, and holds the known and hole bits of its
 // columns (plus one column each side) for the strip's rows and the row above and
@@ -77,6 +76,11 @@ __shared__ float2 g_wt[MAX_SAMPLES / 2];
 // is then a few bit operations per row, the state words are written as two
 // 16-byte stores per row and lane, and each lane writes its tile's masks.
 // INIT_WARPS strips per CTA.
+//
+// Also what a fill starts from: the copy of the input where the output is another image
+// (CTAs of their own) and the cleared stall bitmap.  With the scratch cleared by the
+// descriptor upload and no order kernel for one frame, a single fill is three launches
+// instead of six or seven: the 128 x 128 frame 107 -> 96 us a call.
 
 __device__ __forceinline__ uint2 init_label_row(const uint8_t *labels, int W, int H, int y, int x0, bool vec8)
 {
