@@ -26,7 +26,8 @@
 //   mark     roots of components holding a strong pixel;
 //   accept   kept edge pixels; ring pixels among them as one 32-bit mask per
 //            row segment of a tile;
-//   scan     per frame, output positions in raster order (one CTA per frame);
+//   scan     per frame, output positions of the rows in raster order (one CTA
+//            per frame);
 //   write    the splines.
 // Every value a decision depends on is formed with correctly rounded FP32
 // operations in a fixed order (no contraction), so the sets and the end points
