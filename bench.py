@@ -42,15 +42,15 @@ WORKLOAD = ("batched: 64 frames 1920x1080 RGBA fp32 (seeds 100-163), holes U[0.5
 SEED0, NFRAMES = 100, 64
 
 # DRAM traffic of fill_kernel per filled pixel from the ncu capture of the first 8
-# frames of this batch (dram__bytes_read.sum + dram__bytes_write.sum = 36.384512 MB +
-# 0.675584 MB for 534,164 filled pixels).  It holds only for the kernel sources it
+# frames of this batch (dram__bytes_read.sum + dram__bytes_write.sum = 36.400128 MB +
+# 1.142528 MB for 534,164 filled pixels).  It holds only for the kernel sources it
 # was taken on: with any other source the roofline's traffic is reported as null.
 FILL_TRAFFIC = {
     "sources": {
-        "paper_1611_05319_gb300/csrc/gf_fill.cu": "53f6347da3022ebd284ebd39c39f5e8bfe24cf1baea65842f4d27eb6205363de",
-        "paper_1611_05319_gb300/csrc/gf_internal.cuh": "6594df5bed210caf9ed1e4239994c6eefc103d6780be7b7723193423c4c422f3",
+        "paper_1611_05319_gb300/csrc/gf_fill.cu": "80671a685da344caf21bf2046e2421151579b4095c92070f04a19f120b30c4ef",
+        "paper_1611_05319_gb300/csrc/gf_internal.cuh": "442dc9a24ef0dc2ee3afaa3e8c01651543136e49db9011c270f076b14f281ff2",
     },
-    "bytes_per_filled_px": (36.384512e6 + 0.675584e6) / 534164,
+    "bytes_per_filled_px": (36.400128e6 + 1.142528e6) / 534164,
 }
 
 
