@@ -872,7 +872,7 @@ __device__ __forceinline__ int32_t list_get(const Lists &L, int slot, int pos)
 }
 
 struct WarpCounters {
-    int filled, delta, evals, err, rechecks;
+    int filled, delta, evals, err, rechecks, guided;
 };
 
 // Neighbour-tile claims of step k (tiles for the work list of step k+1).  A claim
@@ -1269,15 +1269,15 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
     }
     const int nr = __popcll(Rm);
     if (phase1) {
-        // guided pixels filled: the data term stays on while any is left
+        // guided pixels filled: the data term stays on while any is left (counted with the
+        // step's fills; a count kept in one place would change under the warps that read it)
         bool gz[2];
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             const int pix = lane + 32 * h;
             gz[h] = ((Rm >> pix) & 1ull) && (ws->guide[pix].x != 0.0f || ws->guide[pix].y != 0.0f);
         }
-        const int ng = __popc(__ballot_sync(FULL, gz[0])) + __popc(__ballot_sync(FULL, gz[1]));
-        if (lane == 0 && ng) atomicSub(F.gleft, ng);
+        wc.guided += __popc(__ballot_sync(FULL, gz[0])) + __popc(__ballot_sync(FULL, gz[1]));
     }
 
     // ---- the fills (state word k: not readable by any other test of step k)
@@ -1349,39 +1349,46 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
 
 __device__ __forceinline__ void clear_step(StepCtl *c)
 {
-    reinterpret_cast<int4 *>(c)[0] = make_int4(0, 0, 0, 0);
-    reinterpret_cast<int4 *>(c)[1] = make_int4(0, 0, 0, 0);
+#pragma unroll
+    for (int i = 0; i < (int)(sizeof(StepCtl) / 16); i++) reinterpret_cast<int4 *>(c)[i] = make_int4(0, 0, 0, 0);
 }
 
-// Adds a warp's counters of step k to slot k%3.  With `clear_next`, lane 0 (of
-// the first warp of each CTA, in a team of the owner's first CTA) also clears
-// the slot of step k+1: its last readers passed the barrier of step k-1 and its
-// next writers start after the barrier of step k.  In a team (`acc` set) the
-// warps add into the CTA's shared counters, which team_sync sends on with one
-// atomic per CTA and counter: 256 warps or more adding to one L2 address would
-// take several microseconds a step.
-__device__ __forceinline__ void flush_counters(GroupCtl *ctl, int *acc, const WarpCounters &wc, int k, bool stall,
+__device__ __forceinline__ PassCtl *pass_ctl(StepCtl *c, int pass)
+{
+    return pass == PASS_EVAL ? &c->eval : &c->later[pass - PASS_AGAIN];
+}
+
+// Adds a warp's counters of a pass of step k to slot k%3.  With `clear_next` (the first
+// warp of the owner's first CTA, in the evaluation pass) lane 0 also clears the slot of
+// step k+1: its last readers passed the barrier of step k-1 and its next writers start
+// after the barrier of step k.  In a team (`acc` set) the warps add into the CTA's
+// shared counters, which team_sync sends on with one atomic per CTA and counter: hundreds
+// of warps adding to one L2 address would take several microseconds a step.
+__device__ __forceinline__ void flush_counters(GroupCtl *ctl, int *acc, const WarpCounters &wc, int k, int pass,
                                                bool clear_next)
 {
     const int lane = threadIdx.x & 31;
     const int s = k % 3;
-    int f = wc.filled, d = wc.delta, e = wc.evals, er = wc.err, rc = wc.rechecks;
+    int f = wc.filled, d = wc.delta, e = wc.evals, er = wc.err, rc = wc.rechecks, gd = wc.guided;
     // all lanes hold identical values except err (per lane)
     er = __reduce_or_sync(FULL, er);
+    if (pass != PASS_EVAL) e = 0;  // Sigma_k |front_k| counts the evaluation pass only
     if (lane == 0) {
         if (acc) {
             if (f) atomicAdd(&acc[0], f);
             if (d) atomicAdd(&acc[1], d);
-            if (e && !stall) atomicAdd(&acc[2], e);
+            if (e) atomicAdd(&acc[2], e);
             if (er) atomicOr(&acc[3], er);
             if (rc) atomicAdd(&acc[4], rc);
+            if (gd) atomicAdd(&acc[5], gd);
         } else {
-            StepCtl *c = &ctl->step[s];
+            PassCtl *c = pass_ctl(&ctl->step[s], pass);
             if (f) atomicAdd(&c->filled, f);
             if (d) atomicAdd(&c->front_delta, d);
-            if (e && !stall) atomicAdd(&c->evals, e);  // Sigma_k |front_k| counts the evaluation pass only
+            if (e) atomicAdd(&c->evals, e);
             if (er) atomicOr(&c->err, er);
             if (rc) atomicAdd(&ctl->rechecks, rc);
+            if (gd) atomicAdd(&ctl->step[s].guided, gd);
         }
         if (clear_next) clear_step(&ctl->step[(k + 1) % 3]);
     }
@@ -1409,6 +1416,7 @@ __device__ __forceinline__ void flush_counters(GroupCtl *ctl, int *acc, const Wa
 // step) 2.94 -> 1.69 ms, a 1500 x 1125 lattice-ball still 2.9 -> 1.8 ms, 32 uneven
 // 1080p frames (on clusters of 4) 4.83 -> 3.90 ms; thin cracks on one 1080p frame,
 // where few steps are that long, 1.32 -> 1.19 ms.
+constexpr int TEAM_COUNTERS = 6;  // a CTA's counters of a pass: filled, front_delta, evals, err; rechecks, guided
 constexpr unsigned TEAM_POLLS = 1u << 22;  // polls (about half a microsecond each) before a wait gives up
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
@@ -1426,18 +1434,19 @@ __device__ __forceinline__ int ld_volatile(const int32_t *p) { return *(const vo
 // Clusters that a step of n tiles keeps busy (`unit` warps each, one tile per warp).
 __device__ __forceinline__ int team_need(int n, int unit) { return n <= unit ? 1 : (n + unit - 1) / unit; }
 
-// The barrier of a team's step (slot = step % 3): sends the CTA's counters, then
-// waits until `target` arrivals have been counted.  False when the wait gave up.
-__device__ __forceinline__ bool team_sync(TeamCtl *tc, int *acc, int *dead, int slot, uint32_t target)
+// The barrier of a pass of a team's step (slot = step % 3): sends the CTA's counters,
+// then waits until `target` arrivals have been counted.  False when the wait gave up.
+__device__ __forceinline__ bool team_sync(TeamCtl *tc, int *acc, int *dead, int slot, int pass, uint32_t target)
 {
     __syncthreads();
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
-        if (lane < 5) {
+        if (lane < TEAM_COUNTERS) {
             const int v = acc[lane];
             acc[lane] = 0;
+            StepCtl *s = &tc->c.step[slot];
             // err is 0 or 1 per CTA: a sum serves as well as an OR
-            if (v) atomicAdd(lane < 4 ? &tc->c.step[slot].filled + lane : &tc->c.rechecks, v);
+            if (v) atomicAdd(lane < 4 ? &pass_ctl(s, pass)->filled + lane : (lane == 4 ? &tc->c.rechecks : &s->guided), v);
         }
         __syncwarp();
         if (lane == 0) {
@@ -1532,7 +1541,7 @@ __device__ __forceinline__ WarpCounters sweep_tiles(const FillParams &p, const F
                                                  const Lists lists, int k, int gw, int nw, bool phase1)
 {
     const int lane = threadIdx.x & 31;
-    WarpCounters wc = {0, 0, 0, 0, 0};
+    WarpCounters wc = {0, 0, 0, 0, 0, 0};
     PendingClaims pc;
     pc.m1 = 0u;
     pc.m2 = 0u;
@@ -1567,7 +1576,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
     __shared__ GroupCtl s_ctl;
     __shared__ int32_t s_lists[3 * DS_LIST];
     __shared__ Role s_role[2];
-    __shared__ int s_acc[5];   // the CTA's step counters while it is in a team
+    __shared__ int s_acc[TEAM_COUNTERS];  // the CTA's step counters while it is in a team
     __shared__ Totals s_tot;   // the leader's
     __shared__ int s_dead;     // a team barrier's wait gave up
     GroupCtl *const ds_ctl = cluster.map_shared_rank(&s_ctl, 0);
@@ -1591,7 +1600,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
         }
     }
     if ((threadIdx.x & 31) == 0) ws->col[WarpSmem<RW>::WS * WarpSmem<RW>::WS] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (threadIdx.x < 5) s_acc[threadIdx.x] = 0;
+    if (threadIdx.x < TEAM_COUNTERS) s_acc[threadIdx.x] = 0;
     if (threadIdx.x == 0) s_dead = 0;
     __syncthreads();
 
@@ -1644,18 +1653,19 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             ctl = team > 1 ? &tc->c : ds_ctl;
             lists.nds = team > 1 ? 0 : DS_LIST;
         };
-        // adds the step's counters and waits for everyone; `leave`: arrivals owed by
+        // adds a pass's counters and waits for everyone; `leave`: arrivals owed by
         // CTAs that left the team at the end of the last step
         int leave = 0;
-        auto finish = [&](const WarpCounters &w, int k, bool stall, bool clear) -> bool {
-            flush_counters(ctl, team > 1 ? s_acc : nullptr, w, k, stall, clear);
+        auto finish = [&](const WarpCounters &w, int k, int pass) -> bool {
+            flush_counters(ctl, team > 1 ? s_acc : nullptr, w, k, pass,
+                           pass == PASS_EVAL && threadIdx.x < 32 && own && crank == 0);
             if (team == 1) {
                 cluster.sync();
                 return true;
             }
             bar += (uint32_t)(team * csize + leave);
             leave = 0;
-            return team_sync(tc, s_acc, &s_dead, k % 3, bar);
+            return team_sync(tc, s_acc, &s_dead, k % 3, pass, bar);
         };
 
         int n_front = 0;
@@ -1669,10 +1679,12 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
         // front pixel with eq. ready (the tracked front was built under phase 1)
         bool phase1 = (p.flags & GF_FLAG_DATA) != 0;
         bool reval = false;
+        int gleft = 0;  // hole pixels with g != 0 left, while phase1 (the same in every thread)
         if (own) {
             n_front = ld(&F.init_count[1]);
             n_cur = ld(&F.init_count[0]);
-            if (phase1 && ld(F.gleft) == 0) {
+            if (phase1) gleft = ld(F.gleft);
+            if (phase1 && gleft == 0) {
                 phase1 = false;
                 if (leader) s_tot.data_switch = 0;
             }
@@ -1685,6 +1697,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             n_front = adm.n_front;
             phase1 = adm.phase1 != 0;
             reval = adm.reval != 0;
+            gleft = adm.gleft;
             bar = adm.bar;
             admitted = adm.first_ticket + (adm.team - adm.first_member);
         }
@@ -1700,6 +1713,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             tc->adm.reval = reval ? 1 : 0;
             tc->adm.bar = bar;
             tc->adm.n_front = n_front;
+            tc->adm.gleft = gleft;
             tc->team = team;
             __threadfence();
             st_release(&tc->admitted, (uint32_t)upto);
@@ -1742,7 +1756,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
         if (gw < n_cur) t0_cur = k == 0 ? ld(&F.init_list[gw]) : list_get(lists, k % 3, gw);
         for (;;) {
             const int slot = k % 3;
-            WarpCounters wc = {0, 0, 0, 0, 0};
+            WarpCounters wc = {0, 0, 0, 0, 0, 0};
             int asked = 0;
             if (leader && open) asked = (int)*(volatile uint32_t *)&tc->want;
             // The leader's own blocks leave its warp in two parts, and without a __syncwarp
@@ -1785,19 +1799,19 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
                 claims_drain(p, ctl, lists, pc, wc);
             }
             if (leader && open) ctl->step[slot].join = asked;
-            if (!finish(wc, k, false, threadIdx.x < 32 && (team == 1 || (own && crank == 0)))) {
+            if (!finish(wc, k, PASS_EVAL)) {
                 status = GF_ERR_TIMEOUT;
                 break;
             }
             // one round trip: this step's counters and the next step's list
             const int s3n = (k + 1) % 3;
-            const int4 c0 = ld(reinterpret_cast<const int4 *>(&ctl->step[slot]));
-            const int2 c1 = ld(reinterpret_cast<const int2 *>(&ctl->step[slot].next));
+            const int4 c0 = ld(reinterpret_cast<const int4 *>(&ctl->step[slot].eval));
+            const int4 c1 = ld(reinterpret_cast<const int4 *>(&ctl->step[slot].next));
             int filled = c0.x, dlt = c0.y, n_next = c1.x;
             const int ev = c0.z, er = c0.w;
             const int join = open ? c1.y : 0;
             int t0_next = gw < p.list_cap ? list_get(lists, s3n, gw) : -1;  // used only if gw < n_next
-            const int gleft = phase1 ? ld(F.gleft) : -1;
+            gleft -= c1.w;
             if (er) {
                 status = GF_ERR_INTERNAL;
                 break;
@@ -1814,13 +1828,14 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
                 phase1 = false;
                 if (leader) s_tot.data_switch = k;
                 const WarpCounters wr = sweep_tiles<RW, REVAL>(p, F, ws, ctl, lists, k, gw, nw, false);
-                if (!finish(wr, k, true, false)) {
+                if (!finish(wr, k, PASS_AGAIN)) {
                     status = GF_ERR_TIMEOUT;
                     break;
                 }
-                filled = ld(&ctl->step[slot].filled);
-                dlt = ld(&ctl->step[slot].front_delta);
-                const int er1 = ld(&ctl->step[slot].err);
+                const int4 c2 = ld(reinterpret_cast<const int4 *>(pass_ctl(&ctl->step[slot], PASS_AGAIN)));
+                filled = c2.x;
+                dlt += c2.y;
+                const int er1 = c2.w;
                 n_next = ld(&ctl->step[slot].next);
                 t0_next = gw < p.list_cap ? list_get(lists, s3n, gw) : -1;
                 if (er1) {
@@ -1837,17 +1852,15 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             int fk = filled;
             if (filled == 0) {
                 if (n_front + dlt == 0) break;  // Algorithm 1: D^(k) exhausted (or the rest unreachable)
-                // stall rule: no front pixel is ready; fill the front isotropically.  The
-                // stall pass adds to the same slot (its counters were zero after the
-                // evaluation pass, except the front delta).
+                // stall rule: no front pixel is ready; fill the front isotropically
                 const WarpCounters ws2 = sweep_tiles<RW, STALL>(p, F, ws, ctl, lists, k, gw, nw, false);
-                if (!finish(ws2, k, true, false)) {
+                if (!finish(ws2, k, PASS_STALL)) {
                     status = GF_ERR_TIMEOUT;
                     break;
                 }
-                const int sf = ld(&ctl->step[slot].filled);
-                const int dlt2 = ld(&ctl->step[slot].front_delta);
-                const int er2 = ld(&ctl->step[slot].err);
+                const int4 c3 = ld(reinterpret_cast<const int4 *>(pass_ctl(&ctl->step[slot], PASS_STALL)));
+                const int sf = c3.x, er2 = c3.w;
+                dlt += c3.y;
                 // the stall fills appended claims to the next step's list
                 n_next = ld(&ctl->step[slot].next);
                 t0_next = gw < p.list_cap ? list_get(lists, s3n, gw) : -1;
@@ -1856,7 +1869,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
                     break;
                 }
                 if (sf == 0) break;  // front pixels with no readable sample at all
-                n_front += dlt2;
+                n_front += dlt;
                 fk = sf;
                 if (leader) s_tot.stalls++;
                 if (leader && F.stall_bits) atomicOr(&F.stall_bits[k >> 5], 1u << (k & 31));

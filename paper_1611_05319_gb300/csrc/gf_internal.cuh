@@ -98,19 +98,31 @@ struct FrameDev {
     int32_t *holes;               // |D_h| (written by the init kernel)
     int32_t *init_list;           // tiles holding part of d_active D^(0)_h (written by the init kernel)
     int32_t *init_count;          // [0] tiles on init_list, [1] |d_active D^(0)_h|
-    int32_t *gleft;               // GF_FLAG_DATA: unfilled hole pixels with g != 0 (init kernel, then fills)
+    int32_t *gleft;               // GF_FLAG_DATA: hole pixels with g != 0 (init kernel)
 };
 
-// The counters of one step: two 16-byte loads after the step's barrier.
-struct alignas(16) StepCtl {
-    int32_t filled;               // fills (evaluation pass, then stall pass if any)
+// The counters of one pass over a step's tiles.
+struct alignas(16) PassCtl {
+    int32_t filled;               // fills
     int32_t front_delta;          // net change of the front size
     int32_t evals;                // front pixels evaluated (evaluation pass only)
     int32_t err;
+};
+
+// The counters of one step: two 16-byte loads after the step's barrier.  What a warp
+// decides by after a barrier is not written again before the next one, in which it
+// takes part itself: a step's later passes (PASS_AGAIN, PASS_STALL) have counters of
+// their own, since a warp that is late would otherwise read the evaluation pass's with
+// fills of theirs and go another way than the rest.  (`next` they add to: it is read
+// again after each.)
+enum { PASS_EVAL = 0, PASS_AGAIN = 1, PASS_STALL = 2 };
+struct alignas(16) StepCtl {
+    PassCtl eval;                 // the evaluation pass
     int32_t next;                 // length of the next step's work list, built by this step's claims
     int32_t join;                 // tickets of the frame's team (TeamCtl::want) seen when the step began
     int32_t cursor;               // hand-out cursor of the items beyond the warp count
-    int32_t pad;
+    int32_t guided;               // GF_FLAG_DATA: fills with g != 0, while the data term is on
+    PassCtl later[2];             // the re-evaluation without the data term; the stall rule
 };
 
 // Per-cluster control block (in the shared memory of the cluster's first CTA,
@@ -134,6 +146,7 @@ struct Admission {
     int32_t phase1, reval;
     uint32_t bar;                 // arrivals that the team's barrier has counted
     int32_t n_front;
+    int32_t gleft;                // unfilled hole pixels with g != 0 (phase1)
 };
 
 // Per-frame control block in global memory for a frame that several clusters
