@@ -44,7 +44,7 @@ typedef enum {
     GF_INCOMPLETE = 1,       /* some hole pixels could never be filled (walled off) */
     GF_ERR_ARG = -1,         /* invalid argument, detected on the host, nothing launched */
     GF_ERR_CUDA = -2,        /* a CUDA runtime call failed */
-    GF_ERR_TIMEOUT = -3,     /* reserved: a bounded device wait gave up */
+    GF_ERR_TIMEOUT = -3,     /* a bounded device wait gave up: the frame's outputs are not complete */
     GF_ERR_NO_PROGRESS = -4, /* the shell loop hit max_shells before finishing */
     GF_ERR_OOM = -5,         /* scratch allocation failed */
     GF_ERR_UNSUPPORTED = -6, /* device is not sm_103 / feature unavailable */
@@ -366,6 +366,14 @@ gf_status gf_fill_backward(gf_ctx *ctx, int n, const gf_adjoint_frame *frames, c
  * legacy default stream only).  Results do not depend on the launch shape.
  */
 gf_status gf_set_launch_config(gf_ctx *ctx, int cluster_size, int n_clusters, int use_graph);
+
+/*
+ * How long thread-block clusters that fill one frame together wait for each other
+ * before they give up: `polls` polls of about half a microsecond; 0 (the default) for
+ * at least two seconds, more for large frames.  Frames whose fill did not end because
+ * of that have GF_ERR_TIMEOUT in their gf_stats; the context stays usable.
+ */
+gf_status gf_set_wait_limit(gf_ctx *ctx, unsigned polls);
 
 /*
  * Split schedule of the batched fill (no counterpart in the paper; a tuning knob

@@ -133,6 +133,11 @@ class Context:
     def set_launch_config(self, cluster_size: int = 0, n_clusters: int = 0, use_graph: bool = True):
         check(lib().gf_set_launch_config(self._h, cluster_size, n_clusters, int(use_graph)), "gf_set_launch_config")
 
+    def set_wait_limit(self, polls: int = 0):
+        """Polls after which clusters that fill one frame together give up waiting for each
+        other (GF_ERR_TIMEOUT in the frame's stats); 0: seconds."""
+        check(lib().gf_set_wait_limit(self._h, int(polls)), "gf_set_wait_limit")
+
     def last_launch(self):
         a, b = C.c_int(), C.c_int()
         check(lib().gf_get_last_launch(self._h, C.byref(a), C.byref(b)), "gf_get_last_launch")

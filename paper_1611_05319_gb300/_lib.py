@@ -25,7 +25,7 @@ STATUS = {0: "ok", 1: "incomplete", -1: "invalid argument", -2: "CUDA error", -3
 # every function declared in include/guidefill.h
 EXPORTS = ["gf_create", "gf_destroy", "gf_status_string", "gf_last_cuda_error", "gf_fill",
            "gf_fill_batched", "gf_fill_batched_ex", "gf_fill_batched_host", "gf_guidance_from_splines", "gf_guidance_batched",
-           "gf_set_launch_config", "gf_get_last_launch", "gf_max_active_clusters", "gf_fill_backward",
+           "gf_set_launch_config", "gf_set_wait_limit", "gf_get_last_launch", "gf_max_active_clusters", "gf_fill_backward",
            "gf_guide_from_angle", "gf_autotune", "gf_fill_noalloc", "gf_set_split", "gf_get_last_split",
            "gf_detect_splines", "gf_detect_splines_batched", "gf_fill_batched_splines"]
 
@@ -110,6 +110,8 @@ def lib() -> C.CDLL:
         L.gf_guidance_batched.restype = C.c_int
         L.gf_set_launch_config.argtypes = [P, C.c_int, C.c_int, C.c_int]
         L.gf_set_launch_config.restype = C.c_int
+        L.gf_set_wait_limit.argtypes = [P, C.c_uint]
+        L.gf_set_wait_limit.restype = C.c_int
         L.gf_get_last_launch.argtypes = [P, C.POINTER(C.c_int), C.POINTER(C.c_int)]
         L.gf_get_last_launch.restype = C.c_int
         L.gf_max_active_clusters.argtypes = [P, C.c_float, C.c_int]

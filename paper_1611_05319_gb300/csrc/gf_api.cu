@@ -38,6 +38,7 @@ struct gf_ctx {
     int cluster_size = 0;
     int n_clusters = 0;
     int use_graph = 1;
+    unsigned wait_limit = 0;      // polls, 0: by the frames' sizes
     int last_cluster_size = 0, last_n_clusters = 0;
     // split schedule (0 = none): the split_m frames with the largest holes go to a
     // second persistent launch of split_nc clusters of split_cs CTAs, beside the
@@ -376,6 +377,13 @@ gf_status gf_set_launch_config(gf_ctx *ctx, int cluster_size, int n_clusters, in
     return GF_OK;
 }
 
+gf_status gf_set_wait_limit(gf_ctx *ctx, unsigned polls)
+{
+    if (!ctx) return GF_ERR_ARG;
+    ctx->wait_limit = polls;
+    return GF_OK;
+}
+
 /* Launch shape used by the last fill call. */
 gf_status gf_get_last_launch(const gf_ctx *ctx, int *cluster_size, int *n_clusters)
 {
@@ -604,6 +612,13 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
     fp.lists = (int32_t *)(A + off_lists);
     fp.lists_by_frame = nc > n - sm ? 1 : 0;
     fp.teams = allow_teams ? (TeamCtl *)(A + off_teams) + sm : nullptr;
+    // Polls before a wait for another cluster gives up.  A wait lasts as long as the
+    // slowest warp's share of a pass, at most the tiles of a sweep dealt to one warp
+    // (tens of microseconds each, two milliseconds if all 64 pixels need the canonical
+    // FP64 sums), so: two seconds and 4096 polls for every such tile.
+    const int64_t most = *std::max_element(ntiles.begin(), ntiles.end()), strip = (int64_t)32 * FILL_WARPS;
+    fp.polls = ctx->wait_limit ? ctx->wait_limit
+                               : (uint32_t)std::min<int64_t>(INT32_MAX, (1 << 22) + 4096 * 32 * ((most - 1) / (strip * cs) + 1));
     build_tab(prm->eps, fp.tab);
     FillParams fpa = fp;  // the second launch: frame_order[0 .. sm)
     fpa.n_frames = sm;
@@ -611,6 +626,8 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
     fpa.frame_cursor = fp.frame_cursor + 1;
     fpa.lists = fp.lists + (size_t)lists_main * 3 * list_cap;
     fpa.lists_by_frame = 0;
+    if (!ctx->wait_limit && scs > 0)
+        fpa.polls = (uint32_t)std::min<int64_t>(INT32_MAX, (1 << 22) + 4096 * 32 * ((most - 1) / (strip * scs) + 1));
     fpa.teams = allow_teams && snc > 1 ? (TeamCtl *)(A + off_teams) : nullptr;
 
     // graph key: everything the enqueued work depends on
@@ -623,6 +640,7 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
     key = fnv(key, &scs, sizeof(scs));
     key = fnv(key, &snc, sizeof(snc));
     key = fnv(key, &n, sizeof(n));
+    key = fnv(key, &fp.polls, sizeof(fp.polls));
     for (int i = 0; i < n; i++) key = fnv(key, &frames[i].rgba, sizeof(void *));
     key = fnv(key, &arena.ptr, sizeof(void *));
 

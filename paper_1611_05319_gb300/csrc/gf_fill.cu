@@ -152,6 +152,14 @@ __global__ void __launch_bounds__(32 * INIT_WARPS, 4) init_kernel(const __grid_c
     }
     const int unit = (b - first) * INIT_WARPS + (threadIdx.x >> 5);
     if (unit >= TH * strips) return;  // warp-uniform
+    if (unit == 0 && lane == 0) {
+        // stands unless the frame's fill ends: a frame that no cluster has taken when
+        // every one of them has left has no other writer
+        gf_stats st = {};
+        st.status = GF_ERR_TIMEOUT;
+        st.data_switch = -1;
+        *F.stats = st;
+    }
     if (F.stall_bits) {
         // the stall bitmap starts at zero: 64 words per unit, the rest with the last one
         const int words = (int)(((int64_t)H * W + 32) / 32);
@@ -1410,14 +1418,24 @@ __device__ __forceinline__ void flush_counters(GroupCtl *ctl, int *acc, const Wa
 //
 // Team barrier: every CTA adds one to a counter and polls it.  About 1 us a step
 // more than the cluster barrier, which is why a team is only as large as its
-// work list.  Measured against one cluster of 16 CTAs per frame, whole calls: a 4K
+// work list.
+//
+// Every wait for another cluster ends after FillParams::polls polls.  A CTA whose wait
+// gave up marks the frame (TeamCtl::dead, which ends the other waits for it) and its
+// cluster (s_dead in every CTA of it), goes to the cluster's next barrier, whichever the
+// other CTAs come to next, and after that barrier they all leave the kernel: a cluster
+// leaves whole, so no barrier counts a CTA that is gone and nobody reads its shared
+// memory.  A cluster that gets no answer to its ticket marks the frame too, since its
+// owner may count on it from now on.  A frame that a dead cluster was needed for ends
+// with GF_ERR_TIMEOUT.
+//
+// Measured against one cluster of 16 CTAs per frame, whole calls: a 4K
 // frame with a 400 x 400 blob (eps 4; first steps of 1,400 to 4,100 tiles on 256
 // warps) 4.47 -> 3.48 ms, a 2000 x 500 onion-order line problem (about 700 tiles a
 // step) 2.94 -> 1.69 ms, a 1500 x 1125 lattice-ball still 2.9 -> 1.8 ms, 32 uneven
 // 1080p frames (on clusters of 4) 4.83 -> 3.90 ms; thin cracks on one 1080p frame,
 // where few steps are that long, 1.32 -> 1.19 ms.
 constexpr int TEAM_COUNTERS = 6;  // a CTA's counters of a pass: filled, front_delta, evals, err; rechecks, guided
-constexpr unsigned TEAM_POLLS = 1u << 22;  // polls (about half a microsecond each) before a wait gives up
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
 {
@@ -1435,8 +1453,10 @@ __device__ __forceinline__ int ld_volatile(const int32_t *p) { return *(const vo
 __device__ __forceinline__ int team_need(int n, int unit) { return n <= unit ? 1 : (n + unit - 1) / unit; }
 
 // The barrier of a pass of a team's step (slot = step % 3): sends the CTA's counters,
-// then waits until `target` arrivals have been counted.  False when the wait gave up.
-__device__ __forceinline__ bool team_sync(TeamCtl *tc, int *acc, int *dead, int slot, int pass, uint32_t target)
+// then waits until `target` arrivals have been counted.  False when this CTA's wait gave
+// up (then `dead` is set in every CTA of the cluster; `lost` is the CTA's own).
+__device__ __forceinline__ bool team_sync(TeamCtl *tc, int *acc, int *lost, int *dead, int slot, int pass,
+                                          uint32_t target, uint32_t polls)
 {
     __syncthreads();
     if (threadIdx.x < 32) {
@@ -1454,16 +1474,21 @@ __device__ __forceinline__ bool team_sync(TeamCtl *tc, int *acc, int *dead, int 
             atomicAdd(&tc->bar, 1u);
             unsigned n = 0;
             while ((int32_t)(ld_acquire(&tc->bar) - target) < 0) {
-                if (++n >= TEAM_POLLS) {
-                    *dead = 1;
+                if (++n >= polls || ((n & 63u) == 0u && ld_volatile(&tc->dead))) {
+                    *lost = 1;
                     break;
                 }
             }
             __threadfence();
+            if (*lost) {
+                *(volatile int32_t *)&tc->dead = 1;
+                cg::cluster_group cluster = cg::this_cluster();
+                for (unsigned r = 0; r < cluster.num_blocks(); r++) *cluster.map_shared_rank(dead, r) = 1;
+            }
         }
     }
     __syncthreads();
-    return *dead == 0;
+    return *lost == 0;
 }
 
 // A frame's statistics, kept by its leader (in shared memory: the other threads need
@@ -1517,7 +1542,7 @@ __device__ int team_find(const FillParams &p, int unit, Role *role)
         if (lane == 0) {
             TeamCtl *tc = &p.teams[bf];
             const uint32_t ticket = atomicAdd(&tc->want, 1u);
-            for (unsigned n = 0; n < TEAM_POLLS; n++) {
+            for (unsigned n = 0;; n++) {
                 if ((int32_t)(ld_acquire(&tc->admitted) - ticket) > 0) {
                     role->adm = tc->adm;
                     role->owner = tc->owner;
@@ -1526,9 +1551,16 @@ __device__ int team_find(const FillParams &p, int unit, Role *role)
                     break;
                 }
                 if (ld_volatile(&tc->load) < 0) break;  // over, or closed
+                if (n >= p.polls) {
+                    *(volatile int32_t *)&tc->dead = 1;
+                    got = -1;
+                    break;
+                }
             }
         }
-        if (__shfl_sync(FULL, got, 0)) return bf;
+        got = __shfl_sync(FULL, got, 0);
+        if (got < 0) return -1;
+        if (got) return bf;
     }
     return -1;
 }
@@ -1578,7 +1610,8 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
     __shared__ Role s_role[2];
     __shared__ int s_acc[TEAM_COUNTERS];  // the CTA's step counters while it is in a team
     __shared__ Totals s_tot;   // the leader's
-    __shared__ int s_dead;     // a team barrier's wait gave up
+    __shared__ int s_lost;     // the CTA's wait at a team barrier gave up
+    __shared__ int s_dead;     // that of a CTA of the cluster did: read after cluster barriers only
     GroupCtl *const ds_ctl = cluster.map_shared_rank(&s_ctl, 0);
     const Role *const ds_role = cluster.map_shared_rank(s_role, 0);
     Lists lists;
@@ -1601,11 +1634,12 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
     }
     if ((threadIdx.x & 31) == 0) ws->col[WarpSmem<RW>::WS * WarpSmem<RW>::WS] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (threadIdx.x < TEAM_COUNTERS) s_acc[threadIdx.x] = 0;
-    if (threadIdx.x == 0) s_dead = 0;
+    if (threadIdx.x == 0) s_lost = s_dead = 0;
     __syncthreads();
 
     for (int it = 0;; it++) {
         cluster.sync();  // everyone is done with the previous frame's counters
+        if (__syncthreads_or(s_dead)) break;
         if (crank == 0 && threadIdx.x < 32) {
             Role *role = &s_role[it & 1];
             int f = 0, help = 0;
@@ -1665,11 +1699,12 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             }
             bar += (uint32_t)(team * csize + leave);
             leave = 0;
-            return team_sync(tc, s_acc, &s_dead, k % 3, pass, bar);
+            return team_sync(tc, s_acc, &s_lost, &s_dead, k % 3, pass, bar, p.polls);
         };
 
         int n_front = 0;
         int status = GF_OK;
+        bool gone = false;  // the cluster leaves (seen after a barrier within the frame)
         int k = 0;
         if (leader) s_tot = Totals{0, 0, 0, 0, -1};
         const int max_shells = F.max_shells;
@@ -1937,6 +1972,11 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
                     for (int i = 0; i < 3; i++) clear_step(&s_ctl.step[i]);
                 for (int i = crank * blockDim.x + threadIdx.x; i < nh; i += csize * blockDim.x) hs[i] = hg[i];
                 cluster.sync();
+                if (__syncthreads_or(s_dead)) {
+                    status = GF_ERR_TIMEOUT;
+                    gone = true;
+                    break;
+                }
             }
             shape();
             t0_cur = gw < n_cur ? list_get(lists, s3n, gw) : -1;
@@ -1959,7 +1999,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             *F.stats = st;
         }
         __syncthreads();
-        if (s_dead) return;  // a wait gave up: no further barrier can be relied on
+        if (gone) break;
     }
     cp_async_wait_all();  // window copies of a last tile that had no candidates
     // no CTA leaves while another may still read its shared memory (the control

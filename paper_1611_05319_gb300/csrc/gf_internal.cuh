@@ -160,6 +160,7 @@ struct alignas(128) TeamCtl {
     int32_t load;                 // 0 not started, > 0 tiles of the coming step, < 0 closed to joins
     int32_t team;                 // clusters filling the frame
     int32_t owner;                // cluster that took the frame from the queue
+    int32_t dead;                 // a cluster's wait gave up: the others' end too
     Admission adm;
 };
 
@@ -169,6 +170,7 @@ struct FillParams {
     double coef64;                // mu^2 / (2 eps^2), FP64 (same expression as the host)
     double c64;
     uint32_t flags;
+    uint32_t polls;               // polls (about half a microsecond each) before a wait for another cluster gives up
     int32_t n_frames;             // frames of this launch: frame_order[order_first .. order_first + n_frames)
     int32_t list_cap;             // capacity of each work list (max ntiles)
     int32_t order_first;
