@@ -161,10 +161,9 @@ __global__ void __launch_bounds__(32 * INIT_WARPS, 4) init_kernel(const __grid_c
         *F.stats = st;
     }
     if (F.stall_bits) {
-        // the stall bitmap starts at zero: 64 words per unit, the rest with the last one
-        const int words = (int)(((int64_t)H * W + 32) / 32);
-        const int end = unit == TH * strips - 1 ? words : min(words, 64 * (unit + 1));
-        for (int w = 64 * unit + lane; w < end; w += 32) F.stall_bits[w] = 0u;
+        // the stall bitmap starts at zero
+        const WordRange r = stall_words((int64_t)H * W, unit, TH * strips);
+        for (int w = r.begin + lane; w < r.end; w += 32) F.stall_bits[w] = 0u;
     }
     const int ty = unit / strips, sx = unit - ty * strips;
     const int tx = sx * 32 + lane;

@@ -27,6 +27,15 @@ __host__ __device__ inline int init_ctas(int TH, int W) {
     const int strips = ((W + 7) / 8 + 31) / 32;
     return (TH * strips + INIT_WARPS - 1) / INIT_WARPS;
 }
+// The words of the stall bitmap (bits 0 .. px) that a strip clears: 64 each, the rest with
+// the last one.  Narrow frames have many more strips than words, up to 2^25 and more.
+struct WordRange {
+    int begin, end;
+};
+__host__ __device__ inline WordRange stall_words(int64_t px, int unit, int units) {
+    const int64_t words = (px + 32) / 32, b = (int64_t)64 * unit;
+    return WordRange{(int)(b < words ? b : words), (int)(unit == units - 1 || b + 64 > words ? words : b + 64)};
+}
 // and, when the output is another image than the input, CTAs that copy COPY_PIXELS
 // colours each
 constexpr int COPY_PIXELS = 32 * INIT_WARPS * 8;
