@@ -34,8 +34,8 @@ class GuidefillFunction(torch.autograd.Function):
         else:
             guides = [g.guide_from_angle(labels[i], mag[i], phi[i]) for i in range(B)]
         # the frames' results are kept for the backward pass; the caller gets a copy to do
-        # with as it likes
-        kept = torch.empty(tuple(rgba.shape[:3]) + (4,), dtype=torch.float32, device=rgba.device)
+        # with as it likes (on the context's device: colours on the CPU are copied there)
+        kept = torch.empty(tuple(rgba.shape[:3]) + (4,), dtype=torch.float32, device=torch.device("cuda", g.device))
         res = g.fill_batched(list(rgba.unbind()), list(labels.unbind()), guides, eps=eps, mu=muf, c=c,
                              out=list(kept.unbind()), stall=True)
         out = kept.clone()
@@ -51,8 +51,9 @@ class GuidefillFunction(torch.autograd.Function):
         B = grad_out.shape[0]
         grad_out = grad_out.contiguous()
         H, W = ctx.res[0].shell.shape
-        grad_rgba = torch.empty((B, H, W, 4), dtype=torch.float32, device=grad_out.device)
-        grad_phi = torch.empty((B, H, W), dtype=torch.float32, device=grad_out.device)
+        dev = torch.device("cuda", g.device)
+        grad_rgba = torch.empty((B, H, W, 4), dtype=torch.float32, device=dev)
+        grad_phi = torch.empty((B, H, W), dtype=torch.float32, device=dev)
         _, _, gmu = g.fill_backward(ctx.res, ctx.guides, list(grad_out.unbind()), eps=ctx.eps, mu=ctx.mu, c=ctx.c,
                                     out=(grad_rgba.unbind(), grad_phi.unbind()))
         grad_mu = gmu.sum()
