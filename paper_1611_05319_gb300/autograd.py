@@ -26,22 +26,24 @@ class GuidefillFunction(torch.autograd.Function):
         g = context(rgba.device.index)
         B = rgba.shape[0]
         muf = float(mu)
-        if 0 < labels.numel() <= _ONE_FIELD and labels.shape == mag.shape == phi.shape:
+        if all(torch.is_tensor(t) and t.shape == rgba.shape[:3] for t in (labels, mag, phi)) and \
+                0 < labels.numel() <= _ONE_FIELD:
             # one field B times as high: the conversion is per pixel
             H, W = labels.shape[1:]
             field = g.guide_from_angle(labels.reshape(B * H, W), mag.reshape(B * H, W), phi.reshape(B * H, W))
             guides = list(field.view(B, H, W, 2).unbind())
-        else:
+        else:  # lists of frames, batches longer than rgba's
             guides = [g.guide_from_angle(labels[i], mag[i], phi[i]) for i in range(B)]
         # the frames' results are kept for the backward pass; the caller gets a copy to do
         # with as it likes (on the context's device: colours on the CPU are copied there)
         kept = torch.empty(tuple(rgba.shape[:3]) + (4,), dtype=torch.float32, device=torch.device("cuda", g.device))
-        res = g.fill_batched(list(rgba.unbind()), list(labels.unbind()), guides, eps=eps, mu=muf, c=c,
+        res = g.fill_batched(list(rgba.unbind()), [labels[i] for i in range(B)], guides, eps=eps, mu=muf, c=c,
                              out=list(kept.unbind()), stall=True)
         out = kept.clone()
         ctx.res = res
         ctx.guides = guides
         ctx.eps, ctx.mu, ctx.c = eps, muf, c
+        ctx.phi_tensor = torch.is_tensor(phi)  # a list of frames has no gradient
         ctx.mu_device = mu.device if torch.is_tensor(mu) else None
         return out
 
@@ -59,7 +61,7 @@ class GuidefillFunction(torch.autograd.Function):
         grad_mu = gmu.sum()
         if ctx.mu_device is not None:
             grad_mu = grad_mu.to(ctx.mu_device)
-        return grad_rgba, None, None, grad_phi, grad_mu, None, None
+        return grad_rgba, None, None, grad_phi if ctx.phi_tensor else None, grad_mu, None, None
 
 
 def guidefill_fill(rgba, labels, mag, phi, mu, eps=3.0, c=0.05):

@@ -47,3 +47,19 @@ def test_colours_on_the_cpu(cuda_device):
     rgba, labels, mag, phi, up = _inputs()
     want = _run(rgba, labels, mag, phi, phi, up)
     _assert_same(_run(rgba.cpu(), labels, mag, phi, phi, up), want)
+
+
+@pytest.mark.parametrize("form", ["lists", "longer", "mixed"])
+def test_labels_and_angles_by_frame(cuda_device, form):
+    """They are taken frame by frame: lists of frames and batches longer than rgba's."""
+    import torch
+    rgba, labels, mag, phi, up = _inputs()
+    rgba.requires_grad_()
+    want = _run(rgba, labels, mag, phi, rgba, up)
+    if form == "lists":
+        labels, mag, phi = list(labels), list(mag), list(phi.detach())
+    elif form == "longer":
+        labels, mag, phi = (torch.cat([t, t[:1]]) for t in (labels, mag, phi.detach()))
+    else:
+        labels, mag = list(labels), torch.cat([mag, mag[:1]])
+    _assert_same(_run(rgba, labels, mag, phi, rgba, up), want)
