@@ -40,6 +40,14 @@ def _ready(t: torch.Tensor, dev: torch.device, dtype: torch.dtype) -> torch.Tens
     return t.to(dev, dtype).contiguous()
 
 
+def _given(t, dev: torch.device, shape) -> torch.Tensor:
+    """``t``, a caller's float32 output tensor that the library writes through its pointer."""
+    if not (torch.is_tensor(t) and t.device == dev and t.dtype is torch.float32 and tuple(t.shape) == shape and
+            t.is_contiguous()):
+        raise ValueError(f"an output must be a contiguous float32 tensor of shape {shape} on {dev}")
+    return t
+
+
 def _zero(ts: Sequence[torch.Tensor]) -> None:
     """Clears tensors of one dtype with one launch (a launch each costs more host time
     than everything else a call does per frame: 8 frames' detection 0.75 -> 0.45 ms)."""
@@ -236,6 +244,12 @@ class Context:
         ``out``: lists of contiguous float32 tensors to write grad_in and grad_phi to."""
         n = len(results)
         dev = torch.device("cuda", self.device)
+        if out is not None:
+            if len(out) != 2 or len(out[0]) != n or len(out[1]) != n:
+                raise ValueError("out must be two lists of one tensor per frame")
+            for i, r in enumerate(results):
+                _given(out[0][i], dev, (*r.shell.shape, 4))
+                _given(out[1][i], dev, tuple(r.shell.shape))
         frames = (_lib.AdjointFrame * n)()
         gi, gp, keep = [], [], []
         gmu = torch.empty((n,), dtype=torch.float32, device=dev)  # cleared by the call
