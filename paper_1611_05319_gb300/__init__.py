@@ -302,9 +302,10 @@ class Context:
         frames = (_lib.SplineFrame * n)()
         outs, keep = [], []
         for i in range(n):
+            # Python numbers are converted straight to the type, which refuses those it cannot hold
+            off = _ready(torch.as_tensor(offsets[i], dtype=torch.int32), dev, torch.int32)
+            P = _ready(torch.as_tensor(pts[i], dtype=torch.float32), dev, torch.float32)
             lab = _ready(labels[i], dev, torch.uint8)
-            off = _ready(torch.as_tensor(offsets[i]), dev, torch.int32)
-            P = _ready(torch.as_tensor(pts[i]), dev, torch.float32)
             H, W = lab.shape
             g = out[i] if out is not None else torch.empty((H, W, 2), dtype=torch.float32, device=dev)
             w = None
