@@ -187,7 +187,9 @@ __device__ __forceinline__ void nearest_segments(const GuideArgs &a, const Splin
         for (int s0 = 0; s0 < cnt; s0 += 32) {
             __syncwarp();  // the previous segments have been read
             // only segments that come within 3 eta of the hole pixels' box matter (one more
-            // px for FP32's rounding, as for the bins): about half of the bin's
+            // px for FP32's rounding, as for the bins): about half of the bin's.  Beyond 2^20
+            // px that is not enough: the end a + v and the distance that decides are each off
+            // by a few 2^-24 of |v| and of the pixel's coordinates.
             bool keep = false;
             int i = 0;
             float4 S0 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -195,7 +197,9 @@ __device__ __forceinline__ void nearest_segments(const GuideArgs &a, const Splin
                 i = __ldg(&F.bin_list[(size_t)b * BIN_CAP + s0 + lane]);
                 S0 = __ldg(reinterpret_cast<const float4 *>(F.segp + i));
                 const float ex = S0.x + S0.z, ey = S0.y + S0.w;
-                keep = !(fmaxf(S0.x, ex) < box.x || fminf(S0.x, ex) > box.y || fmaxf(S0.y, ey) < box.z ||
+                const bool exact = fabsf(S0.z) + fabsf(S0.w) < 1048576.0f && fmaxf(box.y, box.w) < 1048576.0f;
+                keep = !exact ||
+                       !(fmaxf(S0.x, ex) < box.x || fminf(S0.x, ex) > box.y || fmaxf(S0.y, ey) < box.z ||
                          fminf(S0.y, ey) > box.w);
             }
             const unsigned km = __ballot_sync(0xffffffffu, keep);
