@@ -25,7 +25,10 @@
 // per bin: 329 us on 32 frames of 1920 x 1080 (2.7 M hole pixels).  In pairs, with the
 // same CTAs' work dealt to warps, 241 us; with the value evaluated in one place instead
 // of unrolled per pixel, which kept the instruction cache missing, and the strips taken
-// by whichever warp is free, 129 us.
+// by whichever warp is free, 129 us.  Overflowed bins test every point of the frame
+// against the strip's box, 32 at a time; scanned one by one by every warp they had no more
+// warps than strips, and a 512 x 512 frame of 6,000 segments (eta 11) took 8.9 ms (5.8 with
+// a CTA per bin), now 0.93.
 
 #include "gf_internal.cuh"
 
@@ -73,12 +76,14 @@ __global__ void __launch_bounds__(256) bin_kernel(const __grid_constant__ GuideA
         int mid = (lo + hi) >> 1;
         if (__ldg(&F.offsets[mid]) <= i) lo = mid; else hi = mid;
     }
-    if (F.n_splines <= 0 || i + 1 >= F.n_points || i < __ldg(&F.offsets[0]) || i + 1 >= __ldg(&F.offsets[lo + 1]))
-        return;
-    float2 A = __ldg(&F.pts[i]), B = __ldg(&F.pts[i + 1]);
+    const bool starts = F.n_splines > 0 && i + 1 < F.n_points && i >= __ldg(&F.offsets[0]) && i + 1 < __ldg(&F.offsets[lo + 1]);
+    const float2 A = __ldg(&F.pts[i]), B = starts ? __ldg(&F.pts[i + 1]) : A;
     float vx = __fsub_rn(B.x, A.x), vy = __fsub_rn(B.y, A.y);
     float l2 = __fadd_rn(__fmul_rn(vx, vx), __fmul_rn(vy, vy));
-    if (!(l2 > 0.0f)) return;
+    if (!(l2 > 0.0f)) {
+        F.segp[i].il32 = -1.0f;  // no segment starts here (bins that scan every point)
+        return;
+    }
     {
         // FP64 terms of this segment used by every pixel that picks it (same
         // expressions as a per-pixel evaluation, computed once)
@@ -183,64 +188,46 @@ __device__ __forceinline__ void nearest_segments(const GuideArgs &a, const Splin
         best[j] = INFINITY;
         bi[j] = 0x7fffffff;
     }
-    if (cnt <= BIN_CAP) {
-        for (int s0 = 0; s0 < cnt; s0 += 32) {
-            __syncwarp();  // the previous segments have been read
-            // only segments that come within 3 eta of the hole pixels' box matter (one more
-            // px for FP32's rounding, as for the bins): about half of the bin's.  Beyond 2^20
-            // px that is not enough: the end a + v and the distance that decides are each off
-            // by a few 2^-24 of |v| and of the pixel's coordinates.
-            bool keep = false;
-            int i = 0;
-            float4 S0 = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (s0 + lane < cnt) {
-                i = __ldg(&F.bin_list[(size_t)b * BIN_CAP + s0 + lane]);
-                S0 = __ldg(reinterpret_cast<const float4 *>(F.segp + i));
-                const float ex = S0.x + S0.z, ey = S0.y + S0.w;
-                const bool exact = fabsf(S0.z) + fabsf(S0.w) < 1048576.0f && fmaxf(box.y, box.w) < 1048576.0f;
-                keep = !exact ||
-                       !(fmaxf(S0.x, ex) < box.x || fminf(S0.x, ex) > box.y || fmaxf(S0.y, ey) < box.z ||
-                         fminf(S0.y, ey) > box.w);
-            }
-            const unsigned km = __ballot_sync(0xffffffffu, keep);
-            if (keep) {
-                const int pos = __popc(km & ((1u << lane) - 1u));
-                gw->av[pos] = S0;
-                gw->ilid[pos] = make_float2(__ldg(&F.segp[i].il32), __int_as_float(i));
-            }
-            __syncwarp();
-            const int m = __popc(km);
-            for (int s = 0; s < m; s++) {
-                const float4 S = gw->av[s];
-                const float2 t = gw->ilid[s];
-                const int id = __float_as_int(t.y);
-#pragma unroll
-                for (int j = 0; j < P; j++) {
-                    const float d2 = seg_d2(px[j], py[j], S.x, S.y, S.z, S.w, t.x);
-                    if (d2 < best[j] || (d2 == best[j] && id < bi[j])) {
-                        best[j] = d2;
-                        bi[j] = id;
-                    }
-                }
-            }
+    // the bin's list, or every segment of the frame where that overflowed
+    const bool listed = cnt <= BIN_CAP;
+    const int total = listed ? cnt : F.n_points;
+    for (int s0 = 0; s0 < total; s0 += 32) {
+        __syncwarp();  // the previous segments have been read
+        // only segments that come within 3 eta of the hole pixels' box matter (one more
+        // px for FP32's rounding, as for the bins): about half of the bin's.  Beyond 2^20
+        // px that is not enough: the end a + v and the distance that decides are each off
+        // by a few 2^-24 of |v| and of the pixel's coordinates.
+        bool keep = false;
+        int i = 0;
+        float4 S0 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (s0 + lane < total) {
+            i = listed ? __ldg(&F.bin_list[(size_t)b * BIN_CAP + s0 + lane]) : s0 + lane;
+            S0 = __ldg(reinterpret_cast<const float4 *>(F.segp + i));
+            const float ex = S0.x + S0.z, ey = S0.y + S0.w;
+            const bool exact = fabsf(S0.z) + fabsf(S0.w) < 1048576.0f && fmaxf(box.y, box.w) < 1048576.0f;
+            keep = !exact ||
+                   !(fmaxf(S0.x, ex) < box.x || fminf(S0.x, ex) > box.y || fmaxf(S0.y, ey) < box.z ||
+                     fminf(S0.y, ey) > box.w);
+            if (!listed) keep = keep && __ldg(&F.segp[i].il32) >= 0.0f;  // points that start no segment
         }
-    } else {
-        // the bin's list overflowed: every segment of the frame
-        for (int sp = 0; sp < F.n_splines; sp++) {
-            const int i0 = max(0, __ldg(&F.offsets[sp])), i1 = min(F.n_points, __ldg(&F.offsets[sp + 1]));
-            for (int i = i0; i + 1 < i1; i++) {
-                const float2 A = __ldg(&F.pts[i]), B = __ldg(&F.pts[i + 1]);
-                const float vx = __fsub_rn(B.x, A.x), vy = __fsub_rn(B.y, A.y);
-                const float l2 = __fadd_rn(__fmul_rn(vx, vx), __fmul_rn(vy, vy));
-                if (!(l2 > 0.0f)) continue;
-                const float il = __fdiv_rn(1.0f, l2);
+        const unsigned km = __ballot_sync(0xffffffffu, keep);
+        if (keep) {
+            const int pos = __popc(km & ((1u << lane) - 1u));
+            gw->av[pos] = S0;
+            gw->ilid[pos] = make_float2(__ldg(&F.segp[i].il32), __int_as_float(i));
+        }
+        __syncwarp();
+        const int m = __popc(km);
+        for (int s = 0; s < m; s++) {
+            const float4 S = gw->av[s];
+            const float2 t = gw->ilid[s];
+            const int id = __float_as_int(t.y);
 #pragma unroll
-                for (int j = 0; j < P; j++) {
-                    const float d2 = seg_d2(px[j], py[j], A.x, A.y, vx, vy, il);
-                    if (d2 < best[j] || (d2 == best[j] && i < bi[j])) {
-                        best[j] = d2;
-                        bi[j] = i;
-                    }
+            for (int j = 0; j < P; j++) {
+                const float d2 = seg_d2(px[j], py[j], S.x, S.y, S.z, S.w, t.x);
+                if (d2 < best[j] || (d2 == best[j] && id < bi[j])) {
+                    best[j] = d2;
+                    bi[j] = id;
                 }
             }
         }

@@ -30,7 +30,7 @@ struct GuideExp {
 
 // One segment: start a, v = b - a, 1/|v|^2, v/|v|, all but a as pairs, and the spline's
 // weight.  The search for the nearest segment reads the first five numbers (its 1/|v|^2
-// is formed in FP32, il32).
+// is formed in FP32, il32; -1 at points that start no segment).
 struct alignas(16) SegPair {
     float ax, ay, vxh, vyh;
     float il32, vxl, vyl, ilh;
