@@ -612,13 +612,8 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
     fp.lists = (int32_t *)(A + off_lists);
     fp.lists_by_frame = nc > n - sm ? 1 : 0;
     fp.teams = allow_teams ? (TeamCtl *)(A + off_teams) + sm : nullptr;
-    // Polls before a wait for another cluster gives up.  A wait lasts as long as the
-    // slowest warp's share of a pass, at most the tiles of a sweep dealt to one warp
-    // (tens of microseconds each, two milliseconds if all 64 pixels need the canonical
-    // FP64 sums), so: two seconds and 4096 polls for every such tile.
-    const int64_t most = *std::max_element(ntiles.begin(), ntiles.end()), strip = (int64_t)32 * FILL_WARPS;
-    fp.polls = ctx->wait_limit ? ctx->wait_limit
-                               : (uint32_t)std::min<int64_t>(INT32_MAX, (1 << 22) + 4096 * 32 * ((most - 1) / (strip * cs) + 1));
+    const int most_tiles = *std::max_element(ntiles.begin(), ntiles.end());
+    fp.polls = ctx->wait_limit ? ctx->wait_limit : team_polls(most_tiles, cs);
     build_tab(prm->eps, fp.tab);
     FillParams fpa = fp;  // the second launch: frame_order[0 .. sm)
     fpa.n_frames = sm;
@@ -626,8 +621,7 @@ static gf_status enqueue_fill(gf_ctx *ctx, int n, const gf_frame *frames, const 
     fpa.frame_cursor = fp.frame_cursor + 1;
     fpa.lists = fp.lists + (size_t)lists_main * 3 * list_cap;
     fpa.lists_by_frame = 0;
-    if (!ctx->wait_limit && scs > 0)
-        fpa.polls = (uint32_t)std::min<int64_t>(INT32_MAX, (1 << 22) + 4096 * 32 * ((most - 1) / (strip * scs) + 1));
+    if (!ctx->wait_limit && scs > 0) fpa.polls = team_polls(most_tiles, scs);
     fpa.teams = allow_teams && snc > 1 ? (TeamCtl *)(A + off_teams) : nullptr;
 
     // graph key: everything the enqueued work depends on

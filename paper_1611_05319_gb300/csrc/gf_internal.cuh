@@ -173,6 +173,15 @@ struct alignas(128) TeamCtl {
     Admission adm;
 };
 
+// Polls before a wait for another cluster of cs CTAs gives up.  A wait lasts as long as the
+// slowest warp's share of a pass, at most the tiles of a sweep dealt to one warp (tens of
+// microseconds each, two milliseconds if all 64 pixels need the canonical FP64 sums), so:
+// two seconds and 4096 polls for every such tile.
+inline uint32_t team_polls(int64_t tiles, int cs) {
+    const int64_t rounds = (tiles - 1) / ((int64_t)32 * FILL_WARPS * cs) + 1, n = (1 << 22) + 4096 * 32 * rounds;
+    return (uint32_t)(n < INT32_MAX ? n : INT32_MAX);
+}
+
 struct FillParams {
     float eps, mu, c, tau;
     float coef32;                 // mu^2 / (2 eps^2), FP32

@@ -46,10 +46,10 @@ constexpr int64_t NOALLOC_MAX_TILES = 66561;
 constexpr size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 
 struct Layout {
-    size_t U, Q, F, S, L, holes, gleft, icnt, desc, order, cursor, ctaoff, lists, total;
+    size_t U, Q, F, S, L, holes, gleft, icnt, team, desc, order, cursor, ctaoff, lists, total;
 };
 
-// scratch layout of one frame with T tiles, filled by one cluster
+// scratch layout of one frame with T tiles; what starts at zero in one piece, holes to desc
 constexpr Layout layout(int64_t T)
 {
     Layout l{};
@@ -62,6 +62,7 @@ constexpr Layout layout(int64_t T)
     l.holes = p; p = up256(p + 4);
     l.gleft = p; p = up256(p + 4);
     l.icnt = p; p = up256(p + 8);
+    l.team = p; p = up256(p + sizeof(TeamCtl));
     l.desc = p; p = up256(p + sizeof(FrameDev));
     l.order = p; p = up256(p + 4);
     l.cursor = p; p = up256(p + 8);  // two queue heads (order_kernel clears both)
@@ -85,6 +86,7 @@ constexpr int MAX_DEVICES = 64;
 std::mutex g_setup_mutex;
 void *g_scratch_addr[MAX_DEVICES] = {};
 int g_cluster[MAX_DEVICES][3] = {};  // largest schedulable cluster size per window radius 4, 5, 8
+int g_count[MAX_DEVICES][3] = {};    // and how many of it fit at once
 
 int rw_of(float eps)
 {
@@ -119,7 +121,7 @@ cudaError_t setup_device(int dev)
         int best = 0;
         for (int cs = 16; cs >= 1 && best == 0; cs >>= 1) {
             cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(cs);
+            cfg.gridDim = dim3(cs * 64);
             cfg.blockDim = dim3(32 * FILL_WARPS);
             cfg.dynamicSmemBytes = smem_of(rws[i]);
             cudaLaunchAttribute at[1];
@@ -131,7 +133,10 @@ cudaError_t setup_device(int dev)
             cfg.numAttrs = 1;
             int n = 0;
             if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) cudaGetLastError();
-            else if (n > 0) best = cs;
+            else if (n > 0) {
+                best = cs;
+                g_count[dev][i] = n;
+            }
         }
         if (best == 0) return cudaErrorInvalidConfiguration;
         g_cluster[dev][i] = best;
@@ -169,7 +174,14 @@ extern "C" gf_status gf_fill_noalloc(const gf_frame *f, const gf_params *p, gf_s
     const Layout l = layout(T);
     cudaStream_t st = (cudaStream_t)stream;
     const int rw = rw_of(p->eps);
-    const int cs = g_cluster[dev][rw == 4 ? 0 : (rw == 5 ? 1 : 2)];
+    const int kind = rw == 4 ? 0 : (rw == 5 ? 1 : 2);
+    const int cs = g_cluster[dev][kind];
+    // as gf_fill: clusters that join the frame's steps of more tiles than one has warps.  On
+    // one cluster of 192 warps such steps were slower than on the 256 of CTAs of 16 warps:
+    // 1920 x 1080 with bands of 3 to 15 px in onion order 349 us against 325, 179 with teams
+    // (smart order 1154, 948 and 916 us).
+    const int unit = cs * FILL_WARPS;
+    const int nc = std::max(1, std::min(g_count[dev][kind], (int)((T + unit - 1) / unit)));
 
     // ---- descriptor (by value through kernel parameters)
     FrameDev d;
@@ -224,12 +236,13 @@ extern "C" gf_status gf_fill_noalloc(const gf_frame *f, const gf_params *p, gf_s
     fp.frame_order = (int32_t *)(A + l.order);
     fp.frame_cursor = (int32_t *)(A + l.cursor);
     fp.lists = (int32_t *)(A + l.lists);
+    fp.lists_by_frame = 1;
+    fp.teams = nc > 1 ? (TeamCtl *)(A + l.team) : nullptr;
+    fp.polls = team_polls(T, cs);
     build_tab(p->eps, fp.tab);
 
     // ---- clear what must start at zero (the array keeps the last call's contents)
-    if (cudaMemsetAsync(A + l.holes, 0, 4, st) != cudaSuccess) return GF_ERR_CUDA;
-    if (cudaMemsetAsync(A + l.gleft, 0, 4, st) != cudaSuccess) return GF_ERR_CUDA;
-    if (cudaMemsetAsync(A + l.icnt, 0, 8, st) != cudaSuccess) return GF_ERR_CUDA;
+    if (cudaMemsetAsync(A + l.holes, 0, l.desc - l.holes, st) != cudaSuccess) return GF_ERR_CUDA;
     if (f->out_stall && cudaMemsetAsync(f->out_stall, 0, 4 * (((size_t)f->H * f->W + 1 + 31) / 32), st) != cudaSuccess)
         return GF_ERR_CUDA;
     if (f->out_rgba != f->rgba &&
@@ -248,7 +261,7 @@ extern "C" gf_status gf_fill_noalloc(const gf_frame *f, const gf_params *p, gf_s
     order_kernel<<<1, 256, 0, st>>>(fp.frames, 1, fp.frame_order, fp.frame_cursor);
     if (cudaGetLastError() != cudaSuccess) return GF_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)cs);
+    cfg.gridDim = dim3((unsigned)(nc * cs));
     cfg.blockDim = dim3(32 * FILL_WARPS);
     cfg.dynamicSmemBytes = smem_of(rw);
     cfg.stream = st;
