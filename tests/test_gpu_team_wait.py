@@ -60,3 +60,29 @@ def test_short_wait(cuda_device, n, cs, nc, kw):
     finally:
         ctx.set_wait_limit(0)
         ctx.set_launch_config(0, 0)
+
+
+def test_a_cluster_joins_a_running_frame(cuda_device):
+    """Two clusters, two frames: the cluster whose frame ends first joins the other frame in
+    the middle.  With one poll the wait at that team's barrier gives up, so the timeout of the
+    large frame shows that the team was formed."""
+    import torch
+
+    import paper_1611_05319_gb300 as gf
+    ctx = gf.context(0)
+    batch = _batch(1)
+    small = np.zeros((H, W), bool)
+    small[60, 100] = True
+    batch = (batch[0] * 2, batch[1] + [torch.from_numpy(labels_from(small)).cuda()], batch[2] * 2)
+    try:
+        ctx.set_launch_config(16, 1)
+        want = _run(ctx, batch)
+        ctx.set_launch_config(1, 2)
+        assert all(_same(a, b) for a, b in zip(_run(ctx, batch), want))
+        ctx.set_wait_limit(1)
+        got = [_run(ctx, batch) for _ in range(3)]
+        assert any(g[0][0]["status"] == TIMEOUT for g in got)
+        assert all(_same(g[1], want[1]) for g in got)
+    finally:
+        ctx.set_wait_limit(0)
+        ctx.set_launch_config(0, 0)
