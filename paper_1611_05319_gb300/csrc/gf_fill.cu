@@ -1365,8 +1365,9 @@ __device__ __forceinline__ PassCtl *pass_ctl(StepCtl *c, int pass)
     return pass == PASS_EVAL ? &c->eval : &c->later[pass - PASS_AGAIN];
 }
 
-// Adds a warp's counters of a pass of step k to slot k%3.  With `clear_next` (the
-// leader's warp, in the evaluation pass) lane 0 also clears the slot of step k+1: its last readers passed the barrier of step k-1 and its next writers start
+// Adds a warp's counters of a pass of step k to slot k%3.  With `clear_next` (the first
+// warp of the owner's first CTA, in the evaluation pass) lane 0 also clears the slot of
+// step k+1: its last readers passed the barrier of step k-1 and its next writers start
 // after the barrier of step k.  In a team (`acc` set) the warps add into the CTA's
 // shared counters, which team_sync sends on with one atomic per CTA and counter: hundreds
 // of warps adding to one L2 address would take several microseconds a step.
@@ -1661,12 +1662,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
         const int f = role->f;
         if (f < 0) break;
         const bool own = role->help == 0;
-        // The leader is in the first CTA's last warp, which gets work last: a step of few
-        // tiles ends when the first warps' tiles do, and its bookkeeping (statistics,
-        // tickets, the next slot's clearing) beside a tile made a step of one pixel 5.39 us
-        // instead of 5.01 (a 4096-step corridor; 5.53 and 5.26 on eight frames).
-        constexpr int LEADER_WARP = 32 * (FILL_WARPS - 1);
-        const bool leader = own && crank == 0 && threadIdx.x == LEADER_WARP;
+        const bool leader = own && crank == 0 && threadIdx.x == 0;
         if (threadIdx.x == 0) {
             s_frame = p.frames[p.frame_order[p.order_first + f]];
             __threadfence();  // a joining CTA's L1 holds nothing of the frame's earlier steps
@@ -1695,7 +1691,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
         int leave = 0;
         auto finish = [&](const WarpCounters &w, int k, int pass) -> bool {
             flush_counters(ctl, team > 1 ? s_acc : nullptr, w, k, pass,
-                           pass == PASS_EVAL && threadIdx.x >= LEADER_WARP && own && crank == 0);
+                           pass == PASS_EVAL && threadIdx.x < 32 && own && crank == 0);
             if (team == 1) {
                 cluster.sync();
                 return true;
@@ -1798,8 +1794,8 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             int asked = 0;
             if (leader && open) asked = (int)*(volatile uint32_t *)&tc->want;
             // The leader's own blocks leave its warp in two parts, and without a __syncwarp
-            // after each the parts would go through the rest of the step one after the other
-            // (6.7 us a step of one pixel against 5.2 when the leader's warp had the tile).
+            // after each the parts went through the rest of the step one after the other:
+            // 6.7 us a step of one pixel against 5.2 (a 4096-step corridor).
             __syncwarp();
             const bool more = n_cur > nw;
             // lost claims leave markers, up to 1.5 per tile: where they could make the next
