@@ -879,7 +879,7 @@ __device__ __forceinline__ int32_t list_get(const Lists &L, int slot, int pos)
 }
 
 struct WarpCounters {
-    int filled, delta, evals, err, rechecks, guided;
+    int filled, delta, evals, err, rechecks;
 };
 
 // Neighbour-tile claims of step k (tiles for the work list of step k+1).  A claim
@@ -1276,15 +1276,16 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
     }
     const int nr = __popcll(Rm);
     if (phase1) {
-        // guided pixels filled: the data term stays on while any is left (counted with the
-        // step's fills; a count kept in one place would change under the warps that read it)
+        // guided pixels filled: the data term stays on while any is left (counted by step;
+        // a count kept in one place would change under the warps that read it)
         bool gz[2];
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             const int pix = lane + 32 * h;
             gz[h] = ((Rm >> pix) & 1ull) && (ws->guide[pix].x != 0.0f || ws->guide[pix].y != 0.0f);
         }
-        wc.guided += __popc(__ballot_sync(FULL, gz[0])) + __popc(__ballot_sync(FULL, gz[1]));
+        const int ng = __popc(__ballot_sync(FULL, gz[0])) + __popc(__ballot_sync(FULL, gz[1]));
+        if (lane == 0 && ng) atomicAdd(&ctl->step[k % 3].guided, ng);
     }
 
     // ---- the fills (state word k: not readable by any other test of step k)
@@ -1354,50 +1355,60 @@ __device__ void process_tile(const FillParams &p, const FrameDev &F, WarpSmem<RW
     }
 }
 
-__device__ __forceinline__ void clear_step(StepCtl *c)
+// Clears the counters of a step slot.
+__device__ __forceinline__ void clear_step(GroupCtl *ctl, int slot)
 {
-#pragma unroll
-    for (int i = 0; i < (int)(sizeof(StepCtl) / 16); i++) reinterpret_cast<int4 *>(c)[i] = make_int4(0, 0, 0, 0);
+    int4 *c = reinterpret_cast<int4 *>(&ctl->step[slot]), *l = reinterpret_cast<int4 *>(&ctl->later[slot]);
+    c[0] = make_int4(0, 0, 0, 0);
+    c[1] = make_int4(0, 0, 0, 0);
+    l[0] = make_int4(0, 0, 0, 0);
+    l[1] = make_int4(0, 0, 0, 0);
 }
 
-__device__ __forceinline__ PassCtl *pass_ctl(StepCtl *c, int pass)
+// The counters of a pass of the step in `slot`.
+__device__ __forceinline__ PassCtl *pass_ctl(GroupCtl *ctl, int slot, int pass)
 {
-    return pass == PASS_EVAL ? &c->eval : &c->later[pass - PASS_AGAIN];
+    return pass == PASS_EVAL ? &ctl->step[slot].eval : &ctl->later[slot][pass - 1];
 }
 
-// Adds a warp's counters of a pass of step k to slot k%3.  With `clear_next` (the first
-// warp of the owner's first CTA, in the evaluation pass) lane 0 also clears the slot of
-// step k+1: its last readers passed the barrier of step k-1 and its next writers start
-// after the barrier of step k.  In a team (`acc` set) the warps add into the CTA's
-// shared counters, which team_sync sends on with one atomic per CTA and counter: hundreds
-// of warps adding to one L2 address would take several microseconds a step.
+// Adds a warp's counters of a pass of step k to slot k%3.  With `clear_next`, lane 0 (of
+// the first warp of each CTA, in a team of the owner's first CTA) also clears
+// the slot of step k+1: its last readers passed the barrier of step k-1 and its
+// next writers start after the barrier of step k.  In a team (`acc` set) the
+// warps add into the CTA's shared counters, which team_sync sends on with one
+// atomic per CTA and counter: hundreds of warps adding to one L2 address would
+// take several microseconds a step.
+//
+// What is kept between steps matters to the tiles' code: the kernel is at the 168
+// registers that 12 warps leave a thread, and ptxas orders the sample loops' instructions
+// worse with less room.  With the count of guided pixels and the flag of a dead cluster in
+// registers and the waits inline the same instructions took up to 5 % longer (a 4K frame
+// with a blob 3.16 ms, 960 x 1280 at eps 6 660 us, one 1080p frame 1253 us; as here, with
+// both in shared memory and team_sync out of line, 3.06 ms, 637 and 1214 us).
 __device__ __forceinline__ void flush_counters(GroupCtl *ctl, int *acc, const WarpCounters &wc, int k, int pass,
                                                bool clear_next)
 {
     const int lane = threadIdx.x & 31;
     const int s = k % 3;
-    int f = wc.filled, d = wc.delta, e = wc.evals, er = wc.err, rc = wc.rechecks, gd = wc.guided;
+    int f = wc.filled, d = wc.delta, e = wc.evals, er = wc.err, rc = wc.rechecks;
     // all lanes hold identical values except err (per lane)
     er = __reduce_or_sync(FULL, er);
-    if (pass != PASS_EVAL) e = 0;  // Sigma_k |front_k| counts the evaluation pass only
     if (lane == 0) {
         if (acc) {
             if (f) atomicAdd(&acc[0], f);
             if (d) atomicAdd(&acc[1], d);
-            if (e) atomicAdd(&acc[2], e);
+            if (e && pass == PASS_EVAL) atomicAdd(&acc[2], e);
             if (er) atomicOr(&acc[3], er);
             if (rc) atomicAdd(&acc[4], rc);
-            if (gd) atomicAdd(&acc[5], gd);
         } else {
-            PassCtl *c = pass_ctl(&ctl->step[s], pass);
+            PassCtl *c = pass_ctl(ctl, s, pass);
             if (f) atomicAdd(&c->filled, f);
             if (d) atomicAdd(&c->front_delta, d);
-            if (e) atomicAdd(&c->evals, e);
+            if (e && pass == PASS_EVAL) atomicAdd(&c->evals, e);  // Sigma_k |front_k| counts the evaluation pass only
             if (er) atomicOr(&c->err, er);
             if (rc) atomicAdd(&ctl->rechecks, rc);
-            if (gd) atomicAdd(&ctl->step[s].guided, gd);
         }
-        if (clear_next) clear_step(&ctl->step[(k + 1) % 3]);
+        if (clear_next) clear_step(ctl, (k + 1) % 3);
     }
 }
 
@@ -1434,7 +1445,7 @@ __device__ __forceinline__ void flush_counters(GroupCtl *ctl, int *acc, const Wa
 // step) 2.94 -> 1.69 ms, a 1500 x 1125 lattice-ball still 2.9 -> 1.8 ms, 32 uneven
 // 1080p frames (on clusters of 4) 4.83 -> 3.90 ms; thin cracks on one 1080p frame,
 // where few steps are that long, 1.32 -> 1.19 ms.
-constexpr int TEAM_COUNTERS = 6;  // a CTA's counters of a pass: filled, front_delta, evals, err; rechecks, guided
+constexpr int TEAM_COUNTERS = 5;  // a CTA's counters of a pass: filled, front_delta, evals, err; rechecks
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
 {
@@ -1454,7 +1465,7 @@ __device__ __forceinline__ int team_need(int n, int unit) { return n <= unit ? 1
 // The barrier of a pass of a team's step (slot = step % 3): sends the CTA's counters,
 // then waits until `target` arrivals have been counted.  False when this CTA's wait gave
 // up (then `dead` is set in every CTA of the cluster; `lost` is the CTA's own).
-__device__ __forceinline__ bool team_sync(TeamCtl *tc, int *acc, int *lost, int *dead, int slot, int pass,
+__device__ __noinline__ bool team_sync(TeamCtl *tc, int *acc, int *lost, int *dead, int slot, int pass,
                                           uint32_t target, uint32_t polls)
 {
     __syncthreads();
@@ -1463,9 +1474,8 @@ __device__ __forceinline__ bool team_sync(TeamCtl *tc, int *acc, int *lost, int 
         if (lane < TEAM_COUNTERS) {
             const int v = acc[lane];
             acc[lane] = 0;
-            StepCtl *s = &tc->c.step[slot];
             // err is 0 or 1 per CTA: a sum serves as well as an OR
-            if (v) atomicAdd(lane < 4 ? &pass_ctl(s, pass)->filled + lane : (lane == 4 ? &tc->c.rechecks : &s->guided), v);
+            if (v) atomicAdd(lane < 4 ? &pass_ctl(&tc->c, slot, pass)->filled + lane : &tc->c.rechecks, v);
         }
         __syncwarp();
         if (lane == 0) {
@@ -1572,7 +1582,7 @@ __device__ __forceinline__ WarpCounters sweep_tiles(const FillParams &p, const F
                                                  const Lists lists, int k, int gw, int nw, bool phase1)
 {
     const int lane = threadIdx.x & 31;
-    WarpCounters wc = {0, 0, 0, 0, 0, 0};
+    WarpCounters wc = {0, 0, 0, 0, 0};
     PendingClaims pc;
     pc.m1 = 0u;
     pc.m2 = 0u;
@@ -1609,7 +1619,9 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
     __shared__ Role s_role[2];
     __shared__ int s_acc[TEAM_COUNTERS];  // the CTA's step counters while it is in a team
     __shared__ Totals s_tot;   // the leader's
+    __shared__ int s_gleft[FILL_WARPS];  // by warp: hole pixels with g != 0 left, while the data term is on
     __shared__ int s_lost;     // the CTA's wait at a team barrier gave up
+    __shared__ int s_gone;     // the cluster leaves (found at a barrier within a frame)
     __shared__ int s_dead;     // that of a CTA of the cluster did: read after cluster barriers only
     GroupCtl *const ds_ctl = cluster.map_shared_rank(&s_ctl, 0);
     const Role *const ds_role = cluster.map_shared_rank(s_role, 0);
@@ -1633,7 +1645,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
     }
     if ((threadIdx.x & 31) == 0) ws->col[WarpSmem<RW>::WS * WarpSmem<RW>::WS] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (threadIdx.x < TEAM_COUNTERS) s_acc[threadIdx.x] = 0;
-    if (threadIdx.x == 0) s_lost = s_dead = 0;
+    if (threadIdx.x == 0) s_lost = s_dead = s_gone = 0;
     __syncthreads();
 
     for (int it = 0;; it++) {
@@ -1644,7 +1656,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             int f = 0, help = 0;
             if (threadIdx.x == 0) {
                 f = atomicAdd(p.frame_cursor, 1);
-                for (int i = 0; i < 3; i++) clear_step(&s_ctl.step[i]);
+                for (int i = 0; i < 3; i++) clear_step(&s_ctl, i);
                 s_ctl.rechecks = 0;
             }
             f = __shfl_sync(FULL, f, 0);
@@ -1689,9 +1701,8 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
         // adds a pass's counters and waits for everyone; `leave`: arrivals owed by
         // CTAs that left the team at the end of the last step
         int leave = 0;
-        auto finish = [&](const WarpCounters &w, int k, int pass) -> bool {
-            flush_counters(ctl, team > 1 ? s_acc : nullptr, w, k, pass,
-                           pass == PASS_EVAL && threadIdx.x < 32 && own && crank == 0);
+        auto finish = [&](const WarpCounters &w, int k, int pass, bool clear) -> bool {
+            flush_counters(ctl, team > 1 ? s_acc : nullptr, w, k, pass, clear);
             if (team == 1) {
                 cluster.sync();
                 return true;
@@ -1703,7 +1714,6 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
 
         int n_front = 0;
         int status = GF_OK;
-        bool gone = false;  // the cluster leaves (seen after a barrier within the frame)
         int k = 0;
         if (leader) s_tot = Totals{0, 0, 0, 0, -1};
         const int max_shells = F.max_shells;
@@ -1713,12 +1723,11 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
         // front pixel with eq. ready (the tracked front was built under phase 1)
         bool phase1 = (p.flags & GF_FLAG_DATA) != 0;
         bool reval = false;
-        int gleft = 0;  // hole pixels with g != 0 left, while phase1 (the same in every thread)
         if (own) {
             n_front = ld(&F.init_count[1]);
             n_cur = ld(&F.init_count[0]);
-            if (phase1) gleft = ld(F.gleft);
-            if (phase1 && gleft == 0) {
+            if (phase1) s_gleft[threadIdx.x >> 5] = ld(F.gleft);
+            if (phase1 && ld(F.gleft) == 0) {
                 phase1 = false;
                 if (leader) s_tot.data_switch = 0;
             }
@@ -1731,7 +1740,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             n_front = adm.n_front;
             phase1 = adm.phase1 != 0;
             reval = adm.reval != 0;
-            gleft = adm.gleft;
+            s_gleft[threadIdx.x >> 5] = adm.gleft;
             bar = adm.bar;
             admitted = adm.first_ticket + (adm.team - adm.first_member);
         }
@@ -1747,7 +1756,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             tc->adm.reval = reval ? 1 : 0;
             tc->adm.bar = bar;
             tc->adm.n_front = n_front;
-            tc->adm.gleft = gleft;
+            tc->adm.gleft = s_gleft[threadIdx.x >> 5];
             tc->team = team;
             __threadfence();
             st_release(&tc->admitted, (uint32_t)upto);
@@ -1790,7 +1799,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
         if (gw < n_cur) t0_cur = k == 0 ? ld(&F.init_list[gw]) : list_get(lists, k % 3, gw);
         for (;;) {
             const int slot = k % 3;
-            WarpCounters wc = {0, 0, 0, 0, 0, 0};
+            WarpCounters wc = {0, 0, 0, 0, 0};
             int asked = 0;
             if (leader && open) asked = (int)*(volatile uint32_t *)&tc->want;
             // The leader's own blocks leave its warp in two parts, and without a __syncwarp
@@ -1833,19 +1842,25 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
                 claims_drain(p, ctl, lists, pc, wc);
             }
             if (leader && open) ctl->step[slot].join = asked;
-            if (!finish(wc, k, PASS_EVAL)) {
+            if (!finish(wc, k, PASS_EVAL, threadIdx.x < 32 && (team == 1 || (own && crank == 0)))) {
                 status = GF_ERR_TIMEOUT;
                 break;
             }
             // one round trip: this step's counters and the next step's list
             const int s3n = (k + 1) % 3;
             const int4 c0 = ld(reinterpret_cast<const int4 *>(&ctl->step[slot].eval));
-            const int4 c1 = ld(reinterpret_cast<const int4 *>(&ctl->step[slot].next));
+            const int2 c1 = ld(reinterpret_cast<const int2 *>(&ctl->step[slot].next));
             int filled = c0.x, dlt = c0.y, n_next = c1.x;
             const int ev = c0.z, er = c0.w;
             const int join = open ? c1.y : 0;
             int t0_next = gw < p.list_cap ? list_get(lists, s3n, gw) : -1;  // used only if gw < n_next
-            gleft -= c1.w;
+            int gleft = 1;  // hole pixels with g != 0 left
+            if (phase1) {
+                gleft = s_gleft[threadIdx.x >> 5] - ld(&ctl->step[slot].guided);
+                __syncwarp();
+                s_gleft[threadIdx.x >> 5] = gleft;
+                __syncwarp();
+            }
             if (er) {
                 status = GF_ERR_INTERNAL;
                 break;
@@ -1862,14 +1877,13 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
                 phase1 = false;
                 if (leader) s_tot.data_switch = k;
                 const WarpCounters wr = sweep_tiles<RW, REVAL>(p, F, ws, ctl, lists, k, gw, nw, false);
-                if (!finish(wr, k, PASS_AGAIN)) {
+                if (!finish(wr, k, PASS_AGAIN, false)) {
                     status = GF_ERR_TIMEOUT;
                     break;
                 }
-                const int4 c2 = ld(reinterpret_cast<const int4 *>(pass_ctl(&ctl->step[slot], PASS_AGAIN)));
-                filled = c2.x;
-                dlt += c2.y;
-                const int er1 = c2.w;
+                filled = ld(&ctl->later[slot][PASS_AGAIN - 1].filled);
+                dlt += ld(&ctl->later[slot][PASS_AGAIN - 1].front_delta);
+                const int er1 = ld(&ctl->later[slot][PASS_AGAIN - 1].err);
                 n_next = ld(&ctl->step[slot].next);
                 t0_next = gw < p.list_cap ? list_get(lists, s3n, gw) : -1;
                 if (er1) {
@@ -1888,13 +1902,13 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
                 if (n_front + dlt == 0) break;  // Algorithm 1: D^(k) exhausted (or the rest unreachable)
                 // stall rule: no front pixel is ready; fill the front isotropically
                 const WarpCounters ws2 = sweep_tiles<RW, STALL>(p, F, ws, ctl, lists, k, gw, nw, false);
-                if (!finish(ws2, k, PASS_STALL)) {
+                if (!finish(ws2, k, PASS_STALL, false)) {
                     status = GF_ERR_TIMEOUT;
                     break;
                 }
-                const int4 c3 = ld(reinterpret_cast<const int4 *>(pass_ctl(&ctl->step[slot], PASS_STALL)));
-                const int sf = c3.x, er2 = c3.w;
-                dlt += c3.y;
+                const int sf = ld(&ctl->later[slot][PASS_STALL - 1].filled);
+                const int dlt2 = dlt + ld(&ctl->later[slot][PASS_STALL - 1].front_delta);
+                const int er2 = ld(&ctl->later[slot][PASS_STALL - 1].err);
                 // the stall fills appended claims to the next step's list
                 n_next = ld(&ctl->step[slot].next);
                 t0_next = gw < p.list_cap ? list_get(lists, s3n, gw) : -1;
@@ -1903,7 +1917,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
                     break;
                 }
                 if (sf == 0) break;  // front pixels with no readable sample at all
-                n_front += dlt;
+                n_front += dlt2;
                 fk = sf;
                 if (leader) s_tot.stalls++;
                 if (leader && F.stall_bits) atomicOr(&F.stall_bits[k >> 5], 1u << (k & 31));
@@ -1968,12 +1982,12 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
                 if (leader) *(volatile int32_t *)&tc->load = -1;
                 if (member > 0) break;
                 if (leader)
-                    for (int i = 0; i < 3; i++) clear_step(&s_ctl.step[i]);
+                    for (int i = 0; i < 3; i++) clear_step(&s_ctl, i);
                 for (int i = crank * blockDim.x + threadIdx.x; i < nh; i += csize * blockDim.x) hs[i] = hg[i];
                 cluster.sync();
                 if (__syncthreads_or(s_dead)) {
                     status = GF_ERR_TIMEOUT;
-                    gone = true;
+                    if (threadIdx.x == 0) s_gone = 1;
                     break;
                 }
             }
@@ -1998,7 +2012,7 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             *F.stats = st;
         }
         __syncthreads();
-        if (gone) break;
+        if (s_gone) break;
     }
     cp_async_wait_all();  // window copies of a last tile that had no candidates
     // no CTA leaves while another may still read its shared memory (the control

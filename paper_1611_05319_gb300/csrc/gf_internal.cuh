@@ -121,9 +121,9 @@ struct alignas(16) PassCtl {
 // The counters of one step: two 16-byte loads after the step's barrier.  What a warp
 // decides by after a barrier is not written again before the next one, in which it
 // takes part itself: a step's later passes (PASS_AGAIN, PASS_STALL) have counters of
-// their own, since a warp that is late would otherwise read the evaluation pass's with
-// fills of theirs and go another way than the rest.  (`next` they add to: it is read
-// again after each.)
+// their own (GroupCtl::later), since a warp that is late would otherwise read the
+// evaluation pass's with fills of theirs and go another way than the rest.  (`next` they
+// add to: it is read again after each.)
 enum { PASS_EVAL = 0, PASS_AGAIN = 1, PASS_STALL = 2 };
 struct alignas(16) StepCtl {
     PassCtl eval;                 // the evaluation pass
@@ -131,7 +131,6 @@ struct alignas(16) StepCtl {
     int32_t join;                 // tickets of the frame's team (TeamCtl::want) seen when the step began
     int32_t cursor;               // hand-out cursor of the items beyond the warp count
     int32_t guided;               // GF_FLAG_DATA: fills with g != 0, while the data term is on
-    PassCtl later[2];             // the re-evaluation without the data term; the stall rule
 };
 
 // Per-cluster control block (in the shared memory of the cluster's first CTA,
@@ -140,6 +139,7 @@ struct alignas(16) StepCtl {
 // while a warp of the cluster may still read it.
 struct GroupCtl {
     StepCtl step[3];
+    PassCtl later[3][2];          // a step's re-evaluation without the data term, and its stall rule
     int32_t rechecks;             // FP64 re-checks of the current frame (statistics only)
     int32_t pad[3];
 };
