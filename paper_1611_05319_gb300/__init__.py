@@ -243,13 +243,20 @@ class Context:
         ``results`` must come from a fill with ``stall=True`` when it had stall steps.
         ``out``: lists of contiguous float32 tensors to write grad_in and grad_phi to."""
         n = len(results)
-        dev = torch.device("cuda", self.device)
         if out is not None:
+            dev = torch.device("cuda", self.device)
             if len(out) != 2 or len(out[0]) != n or len(out[1]) != n:
                 raise ValueError("out must be two lists of one tensor per frame")
             for i, r in enumerate(results):
                 _given(out[0][i], dev, (*r.shell.shape, 4))
                 _given(out[1][i], dev, tuple(r.shell.shape))
+        return self._backward(results, guides, grad_out, eps, mu, c, smart, snap_tau, max_shells, stream, out)
+
+    def _backward(self, results, guides, grad_out, eps=3.0, mu=50.0, c=0.05, smart=True, snap_tau=1e-5, max_shells=0,
+                  stream=None, out=None):
+        """``fill_backward`` without the checks of ``out`` (a batch's own slices)."""
+        n = len(results)
+        dev = torch.device("cuda", self.device)
         frames = (_lib.AdjointFrame * n)()
         gi, gp, keep = [], [], []
         gmu = torch.empty((n,), dtype=torch.float32, device=dev)  # cleared by the call

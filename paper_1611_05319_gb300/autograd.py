@@ -32,12 +32,14 @@ class GuidefillFunction(torch.autograd.Function):
             H, W = labels.shape[1:]
             field = g.guide_from_angle(labels.reshape(B * H, W), mag.reshape(B * H, W), phi.reshape(B * H, W))
             guides = list(field.view(B, H, W, 2).unbind())
+            labels = labels.unbind()
         else:  # lists of frames, batches longer than rgba's
             guides = [g.guide_from_angle(labels[i], mag[i], phi[i]) for i in range(B)]
+            labels = [labels[i] for i in range(B)]
         # the frames' results are kept for the backward pass; the caller gets a copy to do
         # with as it likes (on the context's device: colours on the CPU are copied there)
         kept = torch.empty(tuple(rgba.shape[:3]) + (4,), dtype=torch.float32, device=torch.device("cuda", g.device))
-        res = g.fill_batched(list(rgba.unbind()), [labels[i] for i in range(B)], guides, eps=eps, mu=muf, c=c,
+        res = g.fill_batched(list(rgba.unbind()), labels, guides, eps=eps, mu=muf, c=c,
                              out=list(kept.unbind()), stall=True)
         out = kept.clone()
         ctx.res = res
@@ -56,8 +58,8 @@ class GuidefillFunction(torch.autograd.Function):
         dev = torch.device("cuda", g.device)
         grad_rgba = torch.empty((B, H, W, 4), dtype=torch.float32, device=dev)
         grad_phi = torch.empty((B, H, W), dtype=torch.float32, device=dev)
-        _, _, gmu = g.fill_backward(ctx.res, ctx.guides, list(grad_out.unbind()), eps=ctx.eps, mu=ctx.mu, c=ctx.c,
-                                    out=(grad_rgba.unbind(), grad_phi.unbind()))
+        _, _, gmu = g._backward(ctx.res, ctx.guides, list(grad_out.unbind()), eps=ctx.eps, mu=ctx.mu, c=ctx.c,
+                                out=(grad_rgba.unbind(), grad_phi.unbind()))
         grad_mu = gmu.sum()
         if ctx.mu_device is not None:
             grad_mu = grad_mu.to(ctx.mu_device)
