@@ -1440,8 +1440,8 @@ __device__ __forceinline__ void flush_counters(GroupCtl *ctl, int *acc, const Wa
 // with GF_ERR_TIMEOUT.
 //
 // Measured against one cluster of 16 CTAs per frame, whole calls: a 4K
-// frame with a 400 x 400 blob (eps 4; first steps of 1,400 to 4,100 tiles on 256
-// warps) 4.47 -> 3.48 ms, a 2000 x 500 onion-order line problem (about 700 tiles a
+// frame with a 400 x 400 blob (eps 4; first steps of 1,400 to 4,100 tiles on the 256
+// warps that a cluster had with CTAs of 16) 4.47 -> 3.48 ms, a 2000 x 500 onion-order line problem (about 700 tiles a
 // step) 2.94 -> 1.69 ms, a 1500 x 1125 lattice-ball still 2.9 -> 1.8 ms, 32 uneven
 // 1080p frames (on clusters of 4) 4.83 -> 3.90 ms; thin cracks on one 1080p frame,
 // where few steps are that long, 1.32 -> 1.19 ms.
@@ -1809,8 +1809,8 @@ __global__ void __launch_bounds__(FILL_WARPS * 32, 1) fill_kernel(const __grid_c
             const bool more = n_cur > nw;
             // lost claims leave markers, up to 1.5 per tile: where they could make the next
             // list longer than the warps, and a second round of it, they are avoided
-            // (a 1080p step of about 180 tiles on 256 warps took 13 us with a list of 400
-            // entries against 9.5 us with a compact one)
+            // (a 1080p step of about 180 tiles on 256 warps, with CTAs of 16, took 13 us with a
+            // list of 400 entries against 9.5 us with a compact one)
             const bool defer = team > 1 || 5 * n_cur > 2 * nw;
             if (rescan) {
                 wc = sweep_tiles<RW, RESCAN>(p, F, ws, ctl, lists, k, gw, nw, phase1);
