@@ -42,15 +42,15 @@ WORKLOAD = ("batched: 64 frames 1920x1080 RGBA fp32 (seeds 100-163), holes U[0.5
 SEED0, NFRAMES = 100, 64
 
 # DRAM traffic of fill_kernel per filled pixel from the ncu capture of the first 8
-# frames of this batch (dram__bytes_read.sum + dram__bytes_write.sum = 36.400128 MB +
-# 1.142528 MB for 534,164 filled pixels).  It holds only for the kernel sources it
+# frames of this batch (dram__bytes_read.sum + dram__bytes_write.sum = 36.410624 MB +
+# 1.092096 MB for 534,164 filled pixels).  It holds only for the kernel sources it
 # was taken on: with any other source the roofline's traffic is reported as null.
 FILL_TRAFFIC = {
     "sources": {
-        "paper_1611_05319_gb300/csrc/gf_fill.cu": "80671a685da344caf21bf2046e2421151579b4095c92070f04a19f120b30c4ef",
-        "paper_1611_05319_gb300/csrc/gf_internal.cuh": "442dc9a24ef0dc2ee3afaa3e8c01651543136e49db9011c270f076b14f281ff2",
+        "paper_1611_05319_gb300/csrc/gf_fill.cu": "5ed322bcaa05d08e5a63d58736a380f27347de2573a4a807ed1391b2f239bfe9",
+        "paper_1611_05319_gb300/csrc/gf_internal.cuh": "2b16627f552ba637d3a8f27bf58fe820352adae1079655f1cc1a1deb31fdb17b",
     },
-    "bytes_per_filled_px": (36.400128e6 + 1.142528e6) / 534164,
+    "bytes_per_filled_px": (36.410624e6 + 1.092096e6) / 534164,
 }
 
 

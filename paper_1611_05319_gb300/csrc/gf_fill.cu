@@ -1439,12 +1439,14 @@ __device__ __forceinline__ void flush_counters(GroupCtl *ctl, int *acc, const Wa
 // owner may count on it from now on.  A frame that a dead cluster was needed for ends
 // with GF_ERR_TIMEOUT.
 //
-// Measured against one cluster of 16 CTAs per frame, whole calls: a 4K
-// frame with a 400 x 400 blob (eps 4; first steps of 1,400 to 4,100 tiles on the 256
-// warps that a cluster had with CTAs of 16) 4.47 -> 3.48 ms, a 2000 x 500 onion-order line problem (about 700 tiles a
-// step) 2.94 -> 1.69 ms, a 1500 x 1125 lattice-ball still 2.9 -> 1.8 ms, 32 uneven
-// 1080p frames (on clusters of 4) 4.83 -> 3.90 ms; thin cracks on one 1080p frame,
-// where few steps are that long, 1.32 -> 1.19 ms.
+// Measured against one cluster of 16 CTAs per frame, whole calls, with the sample loops
+// and the 16 warps per CTA of that time: a 4K frame with a 400 x 400 blob (eps 4; first
+// steps of 1,400 to 4,100 tiles) 4.47 -> 3.48 ms, a 2000 x 500 onion-order line problem
+// (about 700 tiles a step) 2.94 -> 1.69 ms, a 1500 x 1125 lattice-ball still 2.9 -> 1.8 ms,
+// 32 uneven 1080p frames (on clusters of 4) 4.83 -> 3.90 ms; thin cracks on one 1080p
+// frame, where few steps are that long, 1.32 -> 1.19 ms.  Now, one cluster of 192 warps and
+// teams: the 4K frame 4.04 and 3.06 ms, 960 x 1280 at eps 6 807 and 637 us, the line
+// problem 2.58 and 1.22 ms, the still 1.08 and 0.58 ms, the 1080p frame 1.27 and 1.21 ms.
 constexpr int TEAM_COUNTERS = 5;  // a CTA's counters of a pass: filled, front_delta, evals, err; rechecks
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)

@@ -76,7 +76,8 @@ __global__ void __launch_bounds__(256) bin_kernel(const __grid_constant__ GuideA
         int mid = (lo + hi) >> 1;
         if (__ldg(&F.offsets[mid]) <= i) lo = mid; else hi = mid;
     }
-    const bool starts = F.n_splines > 0 && i + 1 < F.n_points && i >= __ldg(&F.offsets[0]) && i + 1 < __ldg(&F.offsets[lo + 1]);
+    const bool starts = F.n_splines > 0 && i + 1 < F.n_points && i >= __ldg(&F.offsets[0]) &&
+                        i + 1 < __ldg(&F.offsets[lo + 1]);
     const float2 A = __ldg(&F.pts[i]), B = starts ? __ldg(&F.pts[i + 1]) : A;
     float vx = __fsub_rn(B.x, A.x), vy = __fsub_rn(B.y, A.y);
     float l2 = __fadd_rn(__fmul_rn(vx, vx), __fmul_rn(vy, vy));
